@@ -1,25 +1,38 @@
 // Hidden 64 -> 64 layers of the learned denoiser on the 5th-generation
-// tensor cores (tcgen05, sm_103a): an implicit GEMM per strip of 128 pixels,
+// tensor cores (tcgen05, sm_103a): an implicit GEMM whose output strips are
+// 128 pixels of one image row,
 //   D[m][co] = sum_{tap, ci} A_tap[m][ci] W[co][tap*64 + ci],
-// M = 128 pixels of one image row, N = 64 output channels, K = 9 x 64.
+// M = 128 pixels, 64 output channels per strip, K = 9 x 64.
 //
 // Operands are K-major with the 128-byte swizzle: a pixel's 64 channels are
 // one 128-byte row, exactly as the activations lie in global memory
 // ([B][H][W][64] BF16), so one TMA copy (box 64 channels x 130 pixels, zero
 // fill outside the image = the convolution's zero padding) brings a whole
-// halo row, and the operand of tap (dy, dx) is the row slot of input row
-// y + dy - 1 started dx rows later.  Weights are staged once per CTA, one 64 x 64
-// block per tap.  A CTA takes a contiguous range of strips, consecutive rows
-// of one 128-column band, so each strip needs one new input row: a ring of
-// NI + 4 row slots keeps the NI + 2 rows that the NI issuing warps' strips
-// read and two loading ahead.  The FP32 accumulators live in tensor memory,
-// two per issuing warp (64 columns each), so the epilogue of one strip
-// (tcgen05.ld, bias + ReLU or the mask, BF16 store) overlaps the MMAs of the
-// next.
+// halo row, and tap column dx of it starts dx rows later.
 //
-// One elected thread per issuing warp issues the 36 MMAs of a strip and commits them to an
-// mbarrier; every wait on it is bounded and reports a timeout through
-// *err instead of hanging.
+// An input row is multiplied once, for all the output rows it touches: image
+// row i gives output row i - 1 its dy = 2 taps, row i its dy = 1 taps and row
+// i + 1 its dy = 0 taps, so with the weights of one dx stacked [dy = 0; 1; 2]
+// one MMA of N = 192 adds into three neighbouring 64-column accumulators.  An
+// MMA of N = 64 is bound by its operand reads (54.6 cycles measured per
+// 128 x 64 x 16, where the arithmetic is 32); N = 192 takes 96.2, which is the
+// arithmetic alone, and reads the pixels once instead of three times.  Every
+// output row still sums its taps in the order dy, dx, ci, as a per-row kernel
+// would, so the results do not depend on the split.
+//
+// A CTA takes a contiguous range of strips, consecutive rows of one
+// 128-column band, and the accumulators of its output rows pass through
+// tensor memory as a ring of eight.  The epilogue (tcgen05.ld, bias + ReLU or
+// the mask, BF16) leaves a strip in shared memory, and one TMA copy stores it.
+//
+// One 512 x 512 layer: 28.3 us with an N = 64 MMA per tap, 19.1 us in this
+// form (ncu; the 17 layers of dgamp_ct_cnn_denoise 512 -> 332 us).  The MMAs
+// used to wait for their issue (see mma_bf16); now a row takes about 1450
+// cycles, of which its 12 MMAs' arithmetic is 1152: the operands (10 KB per
+// MMA), the incoming row and the outgoing strip (twice) share the 128 bytes
+// per cycle of shared memory.
+//
+// Every wait is bounded and reports a timeout through *err instead of hanging.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -35,19 +48,20 @@ constexpr int M = 128;                    // pixels per strip (MMA M)
 constexpr int HWL = M + 2;                // halo pixels loaded per row
 constexpr int HWP = 136;                  // row slot: 136 pixels x 128 B = 17 x 1024 B
 constexpr int A_ROW = HWP * 128;          // bytes of one row slot (pixel-major, 128-byte swizzle)
-constexpr int NI = 4;                     // MMA-issuing warps (strip k goes to warp 1 + k % NI)
-constexpr int RING = NI + 4;              // row slots: NI + 2 rows in use, two loading ahead
+constexpr int RING = 6;                   // row slots: one being multiplied, the others landing
 constexpr int A_BYTES = RING * A_ROW;     // the ring
 constexpr int ROW_BYTES = HWL * 128;      // bytes one row load delivers (130 pixels x 64 channels)
 constexpr int B_TAP = 64 * 128;           // one tap of the weights: 64 co x 64 ci, 128-byte swizzle
-constexpr int B_BYTES = 9 * B_TAP;
-constexpr int SMEM = 1024 + B_BYTES + A_BYTES;       // + alignment slack
-constexpr int EPI_WARP0 = 8;              // warps 8..15: epilogue; warp 0: TMA; warps 1..NI: MMA
+constexpr int B_BYTES = 9 * B_TAP;        // [dx][dy][co][ci]
+constexpr int O_BYTES = M * 128;          // one strip on its way out (and its mask on the way in)
+constexpr int EPI_GROUPS = 2;             // epilogue groups of four warps: group g drains strips k % 2 == g
+constexpr int SMEM = 1024 + B_BYTES + A_BYTES + EPI_GROUPS * O_BYTES;   // + alignment slack
+constexpr int EPI_WARP0 = 4;              // warps 4..11: epilogue; warp 0: TMA; warp 1: MMA
                                           // (the epilogue warps start at a multiple of 4: warp % 4 is
                                           // the TMEM lane quarter a warp may read)
-constexpr int THREADS = 32 * (EPI_WARP0 + 8);
-constexpr int EPI_THREADS = 32 * 8;
-constexpr unsigned TMEM_COLS = 128 * NI;  // 2 NI 64-column FP32 accumulators, two per MMA warp
+constexpr int THREADS = 32 * (EPI_WARP0 + 4 * EPI_GROUPS);
+constexpr int ACCS = 8;                   // ring of 64-column FP32 accumulators
+constexpr unsigned TMEM_COLS = 64 * ACCS;
 constexpr unsigned long long WAIT_NS = 2000000000ull;   // bound of every mbarrier wait (2 s)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -64,22 +78,32 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
            (1ull << 46) | (2ull << 61);
 }
 
-// kind::f16 instruction descriptor: D FP32, A and B BF16, both K-major, N = 64, M = 128
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) |
-                           ((uint32_t)(M >> 4) << 24);
+// kind::f16 instruction descriptor: D FP32, A and B BF16, both K-major, N = 64 count, M = 128
+constexpr uint32_t IDESC0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(M >> 4) << 24);
+__device__ __forceinline__ uint32_t idesc_n(int count) { return IDESC0 | ((uint32_t)(count * (64 >> 3)) << 17); }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+// Called by a whole converged warp; elect.sync picks the one lane that issues
+// (always the same one, so its commits cover its MMAs).  With warp-uniform
+// control flow the operands stay in uniform registers: issued from a branch
+// that only lane 0 takes, the operands are moved there one by one and an MMA
+// took 146 cycles to issue, more than it takes to execute.
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                         uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
         :
-        : "r"(d_tmem), "l"(a), "l"(b), "r"(IDESC), "r"(accumulate));
+        : "r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(mbar)
+        : "memory");
 }
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
@@ -88,12 +112,6 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 
 __device__ __forceinline__ void mbar_init(uint32_t mbar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(mbar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
-    return t;
 }
 
 __device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
@@ -108,15 +126,18 @@ __device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
     return ok != 0;
 }
 
-// Bounded wait for phase `parity` of the mbarrier; false once `bound_ns` has
-// passed.  The clock is read only when the first try fails.
+// Bounded wait for phase `parity` of the mbarrier; false once about `bound_ns`
+// has passed, counted in SM clocks (at most 2.07 per ns; a slower clock only
+// lengthens the bound).  The SM's own counter, because a read of the global
+// timer takes about as long as a strip's arithmetic and every wait of the
+// pipeline that is not satisfied at once would pay for one.
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity,
                                           unsigned long long bound_ns = WAIT_NS) {
     if (mbar_try(mbar, parity)) return true;
-    const unsigned long long t0 = global_ns();
+    const long long t0 = clock64(), bound = 2 * (long long)bound_ns;
     for (;;) {
         if (mbar_try(mbar, parity)) return true;
-        if (global_ns() - t0 > bound_ns) return false;
+        if (clock64() - t0 > bound) return false;
     }
 }
 
@@ -133,12 +154,42 @@ __device__ __forceinline__ void tma_4d(uint32_t dst, const CUtensorMap* map, int
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(mbar)
         : "memory");
 }
-__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t mbar) {
+__device__ __forceinline__ void tma_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, int c4,
+                                       uint32_t mbar) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];\n" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(mbar)
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5, %6}], [%7];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(mbar)
         : "memory");
+}
+
+// TMA tiled store (pixels outside the tensor are dropped), and its group
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+}
+__device__ __forceinline__ void tma_store_read_wait() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
+
+// barrier of `threads` threads (whole warps) of the block
+__device__ __forceinline__ void named_bar(int id, int threads) {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
+}
+
+// 32 consecutive FP32 accumulator columns of this warp's 32 TMEM lanes (no wait)
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+        "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
 }
 
 // 16 consecutive FP32 accumulator columns of this warp's 32 TMEM lanes
@@ -172,128 +223,83 @@ __device__ __forceinline__ Strip strip_of(int s, int H, int nx) {
     return t;
 }
 
-// Input rows in the order the CTA's strips need them: a run of strips of one
-// band needs rows y_first - 1 .. y_last + 1 (rows -1 and H load as zeros);
-// row number q of the sequence goes to ring slot q % RING.
-struct RowCursor {
-    int s_a, s_e;   // current run of strips [s_a, s_e]
-    int y, q;       // next row to load and its sequence number
-    bool done;
-};
-
+// Strips come in runs: the strips [s_a, s_e] of a CTA that lie in one band.  A
+// run needs input rows y(s_a) - 1 .. y(s_e) + 1 (rows -1 and H load as zeros).
 __device__ __forceinline__ int run_end(int s_a, int s1, int H) {
     const int e = (s_a / H + 1) * H;
     return (e < s1 ? e : s1) - 1;
 }
 
-// one input row (130 pixels x 64 channels) -> its ring slot: one TMA copy
-__device__ __forceinline__ void load_row(const CUtensorMap* map, RowCursor& c, int H, int nx, int s1, uint32_t sA,
-                                         uint64_t* row_bar) {
-    const int band = c.s_a / H;
-    const int b = band / nx, x0 = (band - b * nx) * M;
-    const int slot = c.q % RING;
-    const uint32_t bar = smem_u32(&row_bar[slot]);
-    mbar_expect_tx(bar, ROW_BYTES);
-    tma_4d(sA + (uint32_t)(slot * A_ROW), map, 0, x0 - 1, c.y, b, bar);
-    ++c.q;
-    if (++c.y > c.s_e - band * H + 1) {   // past the run's last row + 1: next run
-        c.s_a = c.s_e + 1;
-        if (c.s_a >= s1) {
-            c.done = true;
-        } else {
-            c.s_e = run_end(c.s_a, s1, H);
-            c.y = c.s_a - (c.s_a / H) * H - 1;
-        }
-    }
-}
+// accumulator of a CTA's output row k: descending, so that the rows one input
+// row adds to (newest first) take ascending columns and weight blocks
+__device__ __forceinline__ int acc_of(int k) { return ACCS - 1 - k % ACCS; }
 
-// accumulator of a strip (TMEM columns tcol .. tcol + 63) -> out, with bias +
-// ReLU (MODE 0) or the mask (MODE 1).  Epilogue warp e (warp e + 4) reads TMEM
-// lanes 32 (e % 4) .. +31 (pixels of the strip) and columns 32 (e / 4) .. +31
-// (output channels).
+// Two channels (2j, 2j + 1) of the accumulator columns r: bias + ReLU
+// (MODE 0) or zero where the mask is not positive (MODE 1), rounded to BF16
 template <int MODE>
-__device__ __forceinline__ void epilogue(uint32_t tcol, const Strip& s, int H, int W, const float* __restrict__ bias,
-                                         const bf16* __restrict__ mask, bf16* __restrict__ out, uint32_t empty_bar) {
-    const int ew = (threadIdx.x >> 5) - EPI_WARP0, lane = threadIdx.x & 31;
-    const int quad = ew & 3, c0 = (ew >> 2) * 32;   // quad == warp % 4: the TMEM lanes this warp may read
-    const int x = s.x0 + quad * 32 + lane;
-    const bool live = x < W;
-    const size_t o = (((size_t)s.b * H + s.y) * W + (live ? x : 0)) * CH + c0;
-    const uint32_t taddr = tcol + (uint32_t)c0 + ((uint32_t)(quad * 32) << 16);
-    float v[32];
-    tmem_ld16(taddr, v);          // warp-collective: every lane takes part
-    tmem_ld16(taddr + 16, v + 16);
-    fence_before();               // the reads are complete: the accumulator may be reused
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(empty_bar) : "memory");
-    if (!live) return;
+__device__ __forceinline__ uint32_t finish2(uint32_t r0, uint32_t r1, float2 b, uint32_t mask2) {
+    float v0 = __uint_as_float(r0), v1 = __uint_as_float(r1);
     if (MODE == 0) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i] + __ldg(bias + c0 + i), 0.f);
-    } else {
-        __align__(16) bf16 mk[32];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4*>(mk + 8 * q) = *reinterpret_cast<const uint4*>(mask + o + 8 * q);
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (!(__bfloat162float(mk[i]) > 0.f)) v[i] = 0.f;
+        v0 = fmaxf(v0 + b.x, 0.f);
+        v1 = fmaxf(v1 + b.y, 0.f);
     }
-    __align__(16) __nv_bfloat162 pk[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) pk[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<uint4*>(out + o + 8 * q) = *reinterpret_cast<const uint4*>(pk + 4 * q);
+    __nv_bfloat162 p = __floats2bfloat162_rn(v0, v1);
+    uint32_t o = *reinterpret_cast<uint32_t*>(&p);
+    if (MODE == 1) {
+        const __nv_bfloat162 m = *reinterpret_cast<__nv_bfloat162*>(&mask2);
+        o &= __hgt2_mask(m, __floats2bfloat162_rn(0.f, 0.f));
+    }
+    return o;
 }
-
-// first input-row number of a CTA's strip k given that of strip k - 1: +1
-// inside a band, +3 when strip s starts a new band
-__device__ __forceinline__ int next_q(int Q, int s, int H) { return Q + ((s % H == 0) ? 3 : 1); }
-
-// accumulator of a CTA's strip k: MMA warp k % NI, its own buffer (k / NI) % 2
-__device__ __forceinline__ int acc_of(int k) { return 2 * (k % NI) + ((k / NI) & 1); }
 
 // MODE 0: out = relu(bias + conv(in, Wk)); MODE 1: out = conv(in, Wk) * (mask > 0).
 // stall_ns > 0 is the timeout test: before any copy or MMA is issued, thread 0
 // waits at most stall_ns on an mbarrier that nothing arrives at, records the
 // timeout in *err and the CTA returns without computing (after freeing its
 // tensor memory), exactly as a wait that ran out in the loop reports it.
-// Wk = layer `layer` of a [layers][co][tap*64 + ci] BF16 array (map_w); the
-// input is [B][H][W][64] BF16 (map_in).  CTA k takes strips [k per, (k+1) per).
+// Wk = layer `layer` of a [layers][co][tap*64 + ci] BF16 array (map_w); input,
+// mask and output are [B][H][W][64] BF16.  CTA k takes strips [k per, (k+1) per).
 // Warp-specialised, with no block barrier inside the loop:
 //   warp 0 (one lane): TMA producer -- weights, then input rows into the ring,
-//     a slot refilled once every MMA warp has released its previous row;
-//   warps 1..NI (one lane each): MMA issuers, warp 1 + X for the strips k
-//     with k % NI == X -- one issuing thread cannot feed the tensor core
-//     with N = 64 instructions.  Each waits for its strip's three rows and a
-//     free accumulator of its own, issues 9 taps x 4 channel steps, commits
-//     acc_full, and commits row_empty for every row below its next strip's
-//     first row (each row gets one release from each MMA warp, so a slot is
-//     refilled only after all the MMAs reading it are done);
-//   warps 8..15: epilogue -- wait acc_full, read TMEM, free the accumulator
-//     (acc_empty), then bias + ReLU or mask and the BF16 store.
+//     a slot refilled once the MMAs of its previous row are done;
+//   warp 1 (one lane): MMA issuer -- per input row 12 MMAs (3 dx x 4 channel
+//     steps) over the up to three output rows it touches, then releases the
+//     row's slot and hands over the output row it completes.  The first MMA of
+//     an output row overwrites its accumulator, so it is issued apart;
+//   warps 4..11: epilogue, two groups of four warps on alternate strips --
+//     wait acc_full, read TMEM, free the accumulator (acc_empty), then bias +
+//     ReLU or mask, a lane's pixel as one 128-byte row of the group's buffer
+//     (swizzled, so the eight lanes of a store phase hit distinct banks), and
+//     one TMA store.  The mask of the group's next strip is loaded into the
+//     same buffer once the store has read it: each lane overwrites just the
+//     mask chunk it has read.
 template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
-k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_w, int layer,
-            const float* __restrict__ bias, const bf16* __restrict__ mask, bf16* __restrict__ out, int B, int H,
-            int W, int per, unsigned* err, unsigned long long stall_ns) {
+k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_w,
+            const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_mask, int layer,
+            const float* __restrict__ bias, int B, int H, int W, int per, unsigned* err,
+            unsigned long long stall_ns) {
     extern __shared__ unsigned char smem_raw[];
+    __shared__ __align__(16) float s_bias[CH];
     __shared__ __align__(8) uint64_t row_full[RING];
     __shared__ __align__(8) uint64_t row_empty[RING];
-    __shared__ __align__(8) uint64_t acc_full[2 * NI];
-    __shared__ __align__(8) uint64_t acc_empty[2 * NI];
+    __shared__ __align__(8) uint64_t acc_full[ACCS];
+    __shared__ __align__(8) uint64_t acc_empty[ACCS];
+    __shared__ __align__(8) uint64_t mask_full[EPI_GROUPS];
     __shared__ __align__(8) uint64_t w_bar;
     __shared__ __align__(8) uint64_t never_bar;   // the timeout test's barrier: nothing arrives
     __shared__ uint32_t tmem_slot;
     __shared__ int stalled;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
     const uint32_t raw = smem_u32(smem_raw);
-    const uint32_t sB = (raw + 1023u) & ~1023u, sA = sB + B_BYTES;
+    const uint32_t sB = (raw + 1023u) & ~1023u, sA = sB + B_BYTES, sO = sA + A_BYTES;
     const int nx = (W + M - 1) / M;
     const int nstrips = B * H * nx;
     const int s0 = (int)blockIdx.x * per;
     const int s1 = s0 + per < nstrips ? s0 + per : nstrips;
     if (s0 >= s1) return;
+    pdl_launch();   // the next layer's CTAs set up as soon as this one's shared memory is free
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_slot)),
                      "r"(TMEM_COLS)
@@ -303,21 +309,23 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
     if (tid == 0) {
         for (int r = 0; r < RING; ++r) {
             mbar_init(smem_u32(&row_full[r]), 1);
-            mbar_init(smem_u32(&row_empty[r]), NI);
+            mbar_init(smem_u32(&row_empty[r]), 1);
         }
-        for (int b = 0; b < 2 * NI; ++b) {
+        for (int b = 0; b < ACCS; ++b) {
             mbar_init(smem_u32(&acc_full[b]), 1);
-            mbar_init(smem_u32(&acc_empty[b]), EPI_THREADS);
+            mbar_init(smem_u32(&acc_empty[b]), 4);   // one arrival per warp of the group
         }
+        for (int g = 0; g < EPI_GROUPS; ++g) mbar_init(smem_u32(&mask_full[g]), 1);
         mbar_init(smem_u32(&w_bar), 1);
         mbar_init(smem_u32(&never_bar), 1);
         stalled = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    if (MODE == 0 && tid < CH) s_bias[tid] = bias[tid];
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
     bool ok = true;
     if (stall_ns) {
         if (tid == 0 && !mbar_wait(smem_u32(&never_bar), 0u, stall_ns)) stalled = 1;
@@ -330,82 +338,154 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
         if (lane == 0) {
             // ---- TMA producer ----
             mbar_expect_tx(smem_u32(&w_bar), B_BYTES);
-#pragma unroll 1
-            for (int t = 0; t < 9; ++t) tma_3d(sB + (uint32_t)(t * B_TAP), &map_w, 64 * t, 0, layer, smem_u32(&w_bar));
-            RowCursor cur;
-            cur.s_a = s0;
-            cur.s_e = run_end(s0, s1, H);
-            cur.y = s0 - (s0 / H) * H - 1;
-            cur.q = 0;
-            cur.done = false;
-            while (!cur.done) {
-                const int slot = cur.q % RING;
-                if (cur.q >= RING && !mbar_wait(smem_u32(&row_empty[slot]), (uint32_t)((cur.q / RING - 1) & 1)))
-                    ok = false;
-                load_row(&map_in, cur, H, nx, s1, sA, row_full);
+            tma_5d(sB, &map_w, 0, 0, 0, 0, layer, smem_u32(&w_bar));   // weights: no kernel before this one writes them
+            pdl_wait();   // the input rows are the previous layer's output
+            int q = 0;
+            for (int s_a = s0; s_a < s1;) {
+                const int s_e = run_end(s_a, s1, H);
+                const Strip t = strip_of(s_a, H, nx);
+                for (int i = 0; i < s_e - s_a + 3; ++i, ++q) {
+                    const int slot = q % RING;
+                    if (q >= RING && !mbar_wait(smem_u32(&row_empty[slot]), (uint32_t)((q / RING - 1) & 1))) ok = false;
+                    const uint32_t bar = smem_u32(&row_full[slot]);
+                    mbar_expect_tx(bar, ROW_BYTES);
+                    tma_4d(sA + (uint32_t)(slot * A_ROW), &map_in, 0, t.x0 - 1, t.y - 1 + i, t.b, bar);
+                }
+                s_a = s_e + 1;
             }
         }
-    } else if (warp >= 1 && warp <= NI) {
-        if (lane == 0) {
-            // ---- MMA issuer X for strips k with k % NI == X ----
-            const int X = warp - 1;
-            int q_total = 0;   // input rows of the CTA: first row of the last strip + 3
-            for (int s = s0 + 1; s < s1; ++s) q_total = next_q(q_total, s, H);
-            q_total += 3;
+    } else if (warp == 1) {
+        {
+            // ---- MMA issuer (the whole warp, one elected lane issues) ----
             if (!mbar_wait(smem_u32(&w_bar), 0u)) ok = false;
             const uint64_t bdesc0 = sdesc_sw128(sB);
-            int Q = 0, fx = 0;   // first row of strip k; rows below fx released by this warp
-            int k = 0;
-            for (int s = s0; s < s1; ++s, ++k) {
-                if (k > 0) Q = next_q(Q, s, H);
-                if (k % NI != X) continue;
-                for (; fx < Q; ++fx) mma_commit(smem_u32(&row_empty[fx % RING]));   // rows this warp skips
-                const int a = acc_of(k);
-                if (k >= 2 * NI && !mbar_wait(smem_u32(&acc_empty[a]), (uint32_t)(((k - 2 * NI) / (2 * NI)) & 1)))
-                    ok = false;
-#pragma unroll 1
-                for (int dy = 0; dy < 3; ++dy) {
-                    const int q = Q + dy;
-                    if (!mbar_wait(smem_u32(&row_full[q % RING]), (uint32_t)((q / RING) & 1))) ok = false;
-                }
+            // waits of input row q (ring slot, phase) and, where an output row starts with it, of
+            // that row's accumulator; they run in the middle of the row before, so that the tensor
+            // core still has MMAs queued
+            auto ready = [&](int q, int k, bool fresh) {
+                bool got = true;
+                if (fresh && k >= ACCS) got = mbar_wait(smem_u32(&acc_empty[acc_of(k)]), (uint32_t)((k / ACCS - 1) & 1));
+                got = mbar_wait(smem_u32(&row_full[q % RING]), (uint32_t)((q / RING) & 1)) && got;
+                __syncwarp();
                 fence_after();
-                const uint32_t d = tmem + (uint32_t)(a * 64);
-                // descriptors advance by (byte offset >> 4) in their address field
-                uint64_t arow[3];
+                if (!got) ok = false;
+            };
+            ready(0, 0, true);
+            int q = 0, k0 = 0;   // input row, and the first output row of the run, in the CTA's sequence
+            for (int s_a = s0; s_a < s1;) {
+                const int s_e = run_end(s_a, s1, H), R = s_e - s_a + 1;
+                for (int i = 0; i < R + 2; ++i, ++q) {
+                    const int slot = q % RING;
+                    const int lo = i > 2 ? i - 2 : 0, hi = i < R ? i : R - 1;   // output rows this row adds to
+                    const bool fresh = i < R;                                     // row i starts here (dy = 0)
+                    const uint64_t a0 = sdesc_sw128(sA + (uint32_t)(slot * A_ROW));
+                    // output rows hi, hi - 1, .. lo (accumulators ascending, dy = i - hi ascending) as
+                    // one or, where the accumulator ring wraps, two MMAs
+                    const int first = acc_of(k0 + hi), cnt = hi - lo + 1;
+                    const int n1 = first + cnt > ACCS ? ACCS - first : cnt, n2 = cnt - n1;
+                    const uint32_t d1 = tmem + (uint32_t)(first * 64);
+                    const uint64_t w1 = bdesc0 + (uint64_t)(((i - hi) * B_TAP) >> 4);
+                    const uint64_t w2 = w1 + (uint64_t)((n1 * B_TAP) >> 4);
+                    const uint32_t i1 = idesc_n(n1), i2 = idesc_n(n2);
+                    // first tap (dx = 0, channels 0..15): a fresh row overwrites, the older rows accumulate
+                    mma_bf16(d1, a0, w1, fresh ? idesc_n(1) : i1, fresh ? 0u : 1u);
+                    if (fresh && n1 > 1) mma_bf16(d1 + 64, a0, w1 + (uint64_t)(B_TAP >> 4), idesc_n(n1 - 1), 1u);
+                    if (n2) mma_bf16(tmem, a0, w2, i2, 1u);
+                    // pixel m of the strip reads halo pixel m + dx (dx = t / 4 rows later);
+                    // 16 channels (32 bytes of each row) per MMA
+                    auto taps = [&](int t0, int t1) {
+                        if (n2 == 0) {
 #pragma unroll
-                for (int dy = 0; dy < 3; ++dy) arow[dy] = sdesc_sw128(sA + (uint32_t)(((Q + dy) % RING) * A_ROW));
+                            for (int t = t0; t < t1; ++t)
+                                mma_bf16(d1, a0 + (uint64_t)(((t / 4) * 128 + (t % 4) * 32) >> 4),
+                                         w1 + (uint64_t)(((t / 4) * 3 * B_TAP + (t % 4) * 32) >> 4), i1, 1u);
+                        } else {
 #pragma unroll
-                for (int t = 0; t < 9; ++t) {
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        // pixel m of the strip reads halo pixel m + dx (dx = t % 3 rows later);
-                        // 16 channels (32 bytes of each row) per MMA
-                        const uint64_t ad = arow[t / 3] + (uint64_t)(((t % 3) * 128 + kk * 32) >> 4);
-                        const uint64_t bd = bdesc0 + (uint64_t)((t * B_TAP + kk * 32) >> 4);
-                        mma_bf16(d, ad, bd, (t | kk) != 0 ? 1u : 0u);
-                    }
+                            for (int t = t0; t < t1; ++t) {
+                                const uint64_t ad = a0 + (uint64_t)(((t / 4) * 128 + (t % 4) * 32) >> 4);
+                                const uint64_t wo = (uint64_t)(((t / 4) * 3 * B_TAP + (t % 4) * 32) >> 4);
+                                mma_bf16(d1, ad, w1 + wo, i1, 1u);
+                                mma_bf16(tmem, ad, w2 + wo, i2, 1u);
+                            }
+                        }
+                    };
+                    taps(1, 6);
+                    if (i < R + 1)
+                        ready(q + 1, k0 + i + 1, i + 1 < R);
+                    else if (s_e + 1 < s1)
+                        ready(q + 1, k0 + R, true);
+                    taps(6, 12);
+                    mma_commit(smem_u32(&row_empty[slot]));
+                    if (i >= 2) mma_commit(smem_u32(&acc_full[acc_of(k0 + i - 2)]));
                 }
-                mma_commit(smem_u32(&acc_full[a]));
-                // release the rows below this warp's next strip (strip k + NI)
-                int bound = q_total;
-                if (s + NI < s1) {
-                    bound = Q;
-                    for (int j = 1; j <= NI; ++j) bound = next_q(bound, s + j, H);
-                }
-                for (; fx < bound; ++fx) mma_commit(smem_u32(&row_empty[fx % RING]));
+                k0 += R;
+                s_a = s_e + 1;
             }
-            for (; fx < q_total; ++fx) mma_commit(smem_u32(&row_empty[fx % RING]));
         }
     } else if (warp >= EPI_WARP0) {
         // ---- epilogue ----
-        int k = 0;
-        for (int s = s0; s < s1; ++s, ++k) {
+        const int g = (warp - EPI_WARP0) >> 2, quad = warp & 3;
+        const bool leader = quad == 0 && lane == 0;
+        const uint32_t buf = sO + (uint32_t)(g * O_BYTES);
+        const int pix = quad * 32 + lane;
+        const uint32_t row = buf + (uint32_t)(pix * 128);
+        auto load_mask = [&](int s) {
+            const Strip t = strip_of(s, H, nx);
+            mbar_expect_tx(smem_u32(&mask_full[g]), O_BYTES);
+            tma_4d(buf, &map_mask, 0, t.x0, t.y, t.b, smem_u32(&mask_full[g]));
+        };
+        if (leader) pdl_wait();   // the mask, and the buffer the output replaces, belong to earlier kernels
+        if (MODE == 1 && leader && s0 + g < s1) load_mask(s0 + g);
+        for (int k = g; s0 + k < s1; k += EPI_GROUPS) {
             const int a = acc_of(k);
-            if (!mbar_wait(smem_u32(&acc_full[a]), (uint32_t)((k / (2 * NI)) & 1))) ok = false;
+            if (!mbar_wait(smem_u32(&acc_full[a]), (uint32_t)((k / ACCS) & 1))) ok = false;
+            __syncwarp();
             fence_after();
-            epilogue<MODE>(tmem + (uint32_t)(a * 64), strip_of(s, H, nx), H, W, bias, mask, out,
-                           smem_u32(&acc_empty[a]));
+            uint32_t v[64];
+            const uint32_t taddr = tmem + (uint32_t)(a * 64) + ((uint32_t)(quad * 32) << 16);
+            tmem_ld32(taddr, v);
+            tmem_ld32(taddr + 32, v + 32);
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+            fence_before();               // the reads are complete: the accumulator may be reused
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&acc_empty[a])) : "memory");
+            if (MODE == 1) {
+                if (!mbar_wait(smem_u32(&mask_full[g]), (uint32_t)((k / EPI_GROUPS) & 1))) ok = false;
+            } else {
+                if (leader) tma_store_read_wait();      // the buffer's previous strip has been read
+                named_bar(1 + g, 128);
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {   // 16 bytes = 8 channels, at its swizzled place in the pixel's row
+                const uint32_t at = row + (uint32_t)((c ^ (pix & 7)) * 16);
+                uint32_t m[4] = {0u, 0u, 0u, 0u}, o[4];
+                if (MODE == 1)
+                    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+                                 : "=r"(m[0]), "=r"(m[1]), "=r"(m[2]), "=r"(m[3])
+                                 : "r"(at));
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    float2 b = make_float2(0.f, 0.f);
+                    if (MODE == 0) b = *reinterpret_cast<const float2*>(&s_bias[8 * c + 2 * j]);
+                    o[j] = finish2<MODE>(v[8 * c + 2 * j], v[8 * c + 2 * j + 1], b, m[j]);
+                }
+                asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};\n" ::"r"(at), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                             "r"(o[3])
+                             : "memory");
+            }
+            fence_async_smem();
+            named_bar(1 + g, 128);
+            if (leader) {
+                const Strip t = strip_of(s0 + k, H, nx);
+                tma_store_4d(&map_out, buf, 0, t.x0, t.y, t.b);
+                if (MODE == 1 && s0 + k + EPI_GROUPS < s1) {
+                    tma_store_read_wait();
+                    load_mask(s0 + k + EPI_GROUPS);
+                }
+            }
         }
+        if (leader) tma_store_wait();
     }
     if (!ok && (!stall_ns || tid == 0)) atomicOr(err, 1u);
     fence_before();
@@ -444,15 +524,6 @@ constexpr unsigned WG_TMEM_COLS = 256;                 // three 64-column accumu
 constexpr uint32_t IDESC_WG = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
                               ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(64 >> 4) << 24);
 
-__device__ __forceinline__ void mma_bf16_wg(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        :
-        : "r"(d_tmem), "l"(a), "l"(b), "r"(IDESC_WG), "r"(accumulate));
-}
-
 // MN-major operand, 128-byte swizzle, 64 elements along M or N (one swizzle
 // atom, so the leading-dimension offset is not used): rows of 128 bytes are
 // successive K (pixels), 8-row groups 1024 bytes apart.  The swizzle follows
@@ -473,7 +544,8 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     __shared__ __align__(8) uint64_t never_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int stalled;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
     const int group = blockIdx.x, dy = blockIdx.y;
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t s_base = (raw + 1023u) & ~1023u;
@@ -506,7 +578,7 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
     bool run = true;   // false only in the timeout test: nothing is issued
     if (stall_ns) {
         if (tid == 0 && !mbar_wait(smem_u32(&never_bar), 0u, stall_ns)) stalled = 1;
@@ -533,11 +605,11 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         // every copy issued has landed before the CTA may exit (bounded)
         for (int j = (k > WG_STAGES ? k - WG_STAGES : 0); j < k; ++j)
             if (!mbar_wait(smem_u32(&full[j % WG_STAGES]), (uint32_t)((j / WG_STAGES) & 1))) ok = false;
-    } else if (run && warp == 1 && lane == 0) {
-        // ---- MMA issuer ----
+    } else if (run && warp == 1) {
+        // ---- MMA issuer (the whole warp, one elected lane issues) ----
         for (int k = 0; k < nk; ++k) {
             const int st = k % WG_STAGES;
-            if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((k / WG_STAGES) & 1))) {
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[st]), (uint32_t)((k / WG_STAGES) & 1)))) {
                 ok = false;
                 break;
             }
@@ -549,8 +621,8 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx) {
                     // 16 pixels (rows) per MMA; tap dx reads the halo row dx rows later
-                    mma_bf16_wg(tmem + (uint32_t)(dx * 64), gd + (uint64_t)((ks * 16 * 128) >> 4),
-                                ad + (uint64_t)(((ks * 16 + dx) * 128) >> 4), (k | ks) != 0 ? 1u : 0u);
+                    mma_bf16(tmem + (uint32_t)(dx * 64), gd + (uint64_t)((ks * 16 * 128) >> 4),
+                             ad + (uint64_t)(((ks * 16 + dx) * 128) >> 4), IDESC_WG, (k | ks) != 0 ? 1u : 0u);
                 }
             }
             mma_commit(smem_u32(&empty[st]));
@@ -627,7 +699,7 @@ static int encode(CUtensorMap* map, cuuint32_t rank, const void* base, const cuu
                   const cuuint64_t* strides, const cuuint32_t* box) {
     EncodeTiledFn fn = tensor_map_encoder();
     if (!fn) return cuda_fail(cudaErrorNotSupported);
-    const cuuint32_t es[4] = {1, 1, 1, 1};
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims, strides, box,
                           es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -642,31 +714,29 @@ int launch_conv64_tc(int mode, const void* in, const void* wk_all, int layers, i
     const long long nstrips = (long long)B * H * ((W + tc::M - 1) / tc::M);
     if (nstrips <= 0) return DGAMP_CT_OK;
     if (layer < 0 || layer >= layers) return DGAMP_CT_ERR_INVALID_ARG;
-    CUtensorMap map_in, map_w;
+    CUtensorMap map_in, map_w, map_out, map_mask;
     {
         const cuuint64_t dims[4] = {64, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {128, (cuuint64_t)W * 128, (cuuint64_t)H * W * 128};
         const cuuint32_t box[4] = {64, (cuuint32_t)tc::HWL, 1, 1};
         DGCT_TRY(encode(&map_in, 4, in, dims, strides, box));
+        const cuuint32_t strip[4] = {64, (cuuint32_t)tc::M, 1, 1};
+        DGCT_TRY(encode(&map_out, 4, out, dims, strides, strip));
+        DGCT_TRY(encode(&map_mask, 4, mode == 1 ? mask : in, dims, strides, strip));
     }
     {
-        const cuuint64_t dims[3] = {576, 64, (cuuint64_t)layers};
-        const cuuint64_t strides[2] = {1152, 1152 * 64};
-        const cuuint32_t box[3] = {64, 64, 1};
-        DGCT_TRY(encode(&map_w, 3, wk_all, dims, strides, box));
+        // [layers][co][dy][dx][ci], fetched as [dx][dy][co][ci]
+        const cuuint64_t dims[5] = {64, 64, 3, 3, (cuuint64_t)layers};
+        const cuuint64_t strides[4] = {1152, 384, 128, 1152 * 64};
+        const cuuint32_t box[5] = {64, 64, 3, 3, 1};
+        DGCT_TRY(encode(&map_w, 5, wk_all, dims, strides, box));
     }
     // contiguous ranges of strips, one per CTA, at most grid_cap CTAs
     const int cap = grid_cap > 0 ? grid_cap : 1;
     const int per = (int)((nstrips + cap - 1) / cap);
     const int grid = (int)((nstrips + per - 1) / per);
-    typedef __nv_bfloat16 bf16;
-    if (mode == 0)
-        tc::k_conv64_tc<0><<<grid, tc::THREADS, tc::SMEM, st>>>(map_in, map_w, layer, bias, (const bf16*)mask,
-                                                                (bf16*)out, B, H, W, per, err, stall_ns);
-    else
-        tc::k_conv64_tc<1><<<grid, tc::THREADS, tc::SMEM, st>>>(map_in, map_w, layer, bias, (const bf16*)mask,
-                                                                (bf16*)out, B, H, W, per, err, stall_ns);
-    DGCT_LAUNCH_CHECK();
+    DGCT_CUDA(launch_pdl(mode == 0 ? tc::k_conv64_tc<0> : tc::k_conv64_tc<1>, dim3(grid), dim3(tc::THREADS), tc::SMEM, st,
+                         map_in, map_w, map_out, map_mask, layer, bias, B, H, W, per, err, stall_ns));
     return DGAMP_CT_OK;
 }
 

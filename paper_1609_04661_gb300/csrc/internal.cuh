@@ -336,11 +336,15 @@ int cuda_fail(cudaError_t e);
 // iteration writes (launch parameters, view constants, batch descriptors,
 // the filter), and pdl_wait() returns once every earlier kernel of the
 // stream has completed and its writes are visible.  Nothing the iteration
-// writes is read or written before that.  No kernel signals its dependents
-// early (griddepcontrol.launch_dependents): letting the next kernel's blocks
+// writes is read or written before that.  The iteration's own kernels do not
+// signal their dependents early (griddepcontrol.launch_dependents): letting the next kernel's blocks
 // onto the SMs during a kernel's last wave made the iteration 7% slower,
 // while the launch at completion gains about 1%.  pdl_wait() is a no-op for
 // a kernel launched the ordinary way.
+// pdl_launch() is for kernels whose blocks each fill an SM (the tensor-core
+// convolution): the next kernel's blocks then only enter an SM this kernel has
+// left, and their set-up overlaps the end of the others.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
 inline cudaError_t launch_pdl_c(const void* kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
