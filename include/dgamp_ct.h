@@ -229,9 +229,12 @@ typedef struct {
                              the geometry allows and keeps the faster; filter_mode alone
                              governs the single-step entry points */
     int32_t bp_mode;      /* A^T: 0 = pixel-driven gather (each pixel finds the <= 2 rays
-                             of a view that tap it), 1 = ray-driven over 16 x 16 image
-                             tiles with per-warp shared-memory accumulators.  Both are the
-                             exact transpose of the projector and deterministic */
+                             of a view that tap it and takes the projector's own weights),
+                             1 = 16 x 16 image tiles that stage the rays of 64 views in
+                             shared memory and evaluate the weights from each pixel's
+                             detector coordinate (within 2^-22 of the projector's).  Both
+                             are the projector's transpose and deterministic; a fan-beam
+                             plan's form 1 is ray-driven, with the projector's weights */
     int32_t pj_seg;       /* A: warps that split the step range of one group of 32 rays,
                              8, 16 or 32 (the partial sums are added in a fixed order) */
     int32_t tv_vrows;     /* rows of the TV region each thread holds: 4; 8 or 2 (then the

@@ -98,6 +98,11 @@ static void view_constants(int n, int nd, const std::vector<double>& ang, std::v
         v.PDET = (long long)std::llround(ad * q);
         v.AP = v.PDET > 0 ? v.PDET : -v.PDET;
         v.sg = v.PDET > 0 ? 1 : -1;
+        // d = X cos + Y sin + cd with X = ix - c, Y = c - iy
+        const double q40 = 1099511627776.0;
+        v.Q0 = (long long)std::llround((c * (st - ct) + cd) * q40);
+        v.QX = (long long)std::llround(ct * q40);
+        v.QY = (long long)std::llround(-st * q40);
         out[k] = v;
     }
 }

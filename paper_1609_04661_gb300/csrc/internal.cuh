@@ -28,6 +28,7 @@ constexpr int kBatchStreams = 16;  // streams a batched solve spreads its slices
 struct ViewConst {
     long long P0, PSTEP, PDET;    // a0, a_step, a_det scaled by 2^32
     long long AP;                 // |PDET|: ray spacing on a march line (>= 2^32)
+    long long Q0, QX, QY;         // detector coordinate of pixel (ix, iy): Q0 + ix QX + iy QY, scaled by 2^40
     float a0, a_step, a_det, w;   // w = path length per step (1/|sin| or 1/|cos|)
     float inv_adet;               // 1 / a_det
     int col;                      // 1: march over columns, interpolate along rows

@@ -7,6 +7,8 @@
 // XR, one that marches over columns reads XC, so in both cases a warp of
 // adjacent rays reads adjacent floats of one line per step, and taps that
 // fall just outside the image read zeros instead of being bounds-checked.
+#include <climits>
+
 #include "internal.cuh"
 
 namespace dgct {
@@ -428,65 +430,154 @@ k_backproject(const T* __restrict__ sino, int nv, int nd, int n,
     if (tid == 0) atomicMax(&S->rmax_bits, s_max);
 }
 
-// Ray-driven form of the same transpose (bp_mode 1).  One block = one
-// kBtS x kBtS image tile; warp w takes views w, w + 8, ...  For each view it
-// marches the rays that have a tap in the tile, 32 rays at a time, over the
-// tile's steps with the projector's own fixed-point positions, and adds
-// (1 - f) v w at the left tap into one accumulator tile and f v w at the
-// right tap into a second one (both the warp's own).  On one march line the
-// rays' left taps are distinct (rays are >= 1 apart), and so are their right
-// taps, so no two lanes of a warp ever add to the same word of one
-// accumulator in the same step.  The warps' tiles are summed in a fixed
-// order, so the result does not depend on scheduling.
-constexpr int kBtS = 16, kBtLd = kBtS + 1, kBtWarps = 8;
-
-// One view's rays over the tile.  COL = 1: the view marches over columns
-// (step k = column s0 + k, taps along rows), else over rows.
-template <int COL, typename T>
-__device__ __forceinline__ void bp_tile_view(const ViewConst& c, const T* __restrict__ row, int nd, int n,
-                                             int tx0, int ty0, float* __restrict__ AL, float* __restrict__ AR) {
-    constexpr int as = COL ? 1 : kBtLd, ac = COL ? kBtLd : 1;     // accumulator strides: step, tap
-    const int lane = threadIdx.x & 31;
-    const int s0 = COL ? tx0 : ty0, c0 = COL ? ty0 : tx0;
-    const int ns = min(kBtS, n - s0), nc = min(kBtS, n - c0);
-    // rays with a left tap in [c0 - 1, c0 + nc) at a step of [s0, s0 + ns),
-    // i.e. a0 + d a_det + s a_step in [c0 - 1, c0 + nc): solved for d in
-    // float and widened by one ray on each side
-    const float e0 = (float)s0 * c.a_step, e1 = (float)(s0 + ns - 1) * c.a_step;
-    const float dA = ((float)(c0 - 1) - fmaxf(e0, e1) - c.a0) * c.inv_adet;
-    const float dB = ((float)(c0 + nc) - fminf(e0, e1) - c.a0) * c.inv_adet;
-    const int dlo = max(0, (int)floorf(fminf(dA, dB)) - 1);
-    const int dhi = min(nd - 1, (int)ceilf(fmaxf(dA, dB)) + 1);
-    for (int d0 = dlo; d0 <= dhi; d0 += 32) {
-        const int d = d0 + lane;
-        const float vw = d <= dhi ? ldf(row + d) * c.w : 0.f;        // rays past dhi add zeros
-        // positions relative to the tile: the left tap's index in the tile is the high word
-        long long pos = joseph_pos(c, d, s0) - ((long long)c0 << 32);
-        auto step = [&](int k) {
-            const int rel = (int)(pos >> 32);
-            const float f = __uint_as_float(0x3F800000u | ((unsigned)pos >> 9)) - 1.0f;
-            const int at = k * as + rel * ac;
-            if ((unsigned)rel < (unsigned)nc) AL[at] += (1.f - f) * vw;
-            if ((unsigned)(rel + 1) < (unsigned)nc) AR[at + ac] += f * vw;
-            pos += c.PSTEP;
-        };
-        if (ns == kBtS) {
-#pragma unroll
-            for (int k = 0; k < kBtS; ++k) step(k);
-        } else {
-            for (int k = 0; k < ns; ++k) step(k);
-        }
-    }
-}
+// Tile form of the same transpose (bp_mode 1).  One block = one kBtS x kBtS
+// image tile.  On a march line the rays of a view are A = |a_det| in
+// [1, sqrt 2] pixels apart, so a pixel at detector coordinate q (q = d where
+// ray d passes through its centre) is tapped by rays floor(q) and
+// floor(q) + 1 alone, with Joseph's weights 1 - A (q - d) and
+// 1 - A (d + 1 - q), clamped at 0.  q is linear in the pixel, so a view costs
+// a pixel one fixed-point add, two saturating FMAs for the weights, one
+// 8-byte read of the ray pair and two FMAs: about 10 instructions, where
+// marching the rays through per-warp accumulator tiles took 44 (22.7 M warp
+// instructions at 512^2/64/729, issue-bound).
+//
+// Positions are 5.27 fixed point relative to the tile: the tile's detector
+// coordinate comes from the view's 64-bit constants (units of 2^-40 bins), so
+// only the offsets inside the tile round (8 pixels at 2^-28 each).  The weights
+// then lie within 2^-22 of the projector's, which truncates its fraction to
+// 23 bits.  Rays of the views are staged kBtViews views at a time as pairs
+// (v[d] w, v[d + 1] w); a lane reads 16 consecutive pixels' pairs, at most
+// one apart, without bank conflicts.  Views are summed in order, in partial
+// sums of kBtUnroll, by one thread per pixel pair, so the result does not
+// depend on scheduling.  Per iteration of the 512^2/64/729 solve about 30.7 ->
+// 16 us; one call at 1024^2/90/1449 124 -> about 59 us.  What is left is issue
+// (half of the cycles) and the set-up and staging of blocks that all start at
+// once.  8 blocks per SM: 10 spill, 6 are slower.
+constexpr int kBtS = 16;
+constexpr int kBtWork = 128;                  // threads that take pixels (two each)
+constexpr int kBtThreads = kBtWork + 32;      // and a warp that forms tau_r meanwhile
+constexpr int kBtViews = 64;     // views staged at a time (16 KB)
+constexpr int kBtSlots = 32;     // ray pairs a view can need: 16 (|cos| + |sin|) + 3 < 27
+constexpr int kBtUnroll = 8;
+constexpr int kBtFrac = 27;      // fraction bits of a tile-relative position
+constexpr int kQFrac = 40;       // fraction bits of ViewConst's Q0, QX, QY
 
 struct BtShared {
-    float accL[kBtWarps][kBtS * kBtLd], accR[kBtWarps][kBtS * kBtLd];
+    float2 seg[kBtViews][kBtSlots];
+    int4 vc[kBtViews];           // position of pixel (8, 8), its steps along x and y, and A
+    float2 a12[kBtViews];        // 1 + A, 1 - 2 A
+    float2 low[kBtViews];        // first staged ray (int bits), path length per step
     unsigned s_max;
     float s_tau_r;
 };
 
+// Constants of views v0 .. v0 + cnt - 1 for the tile at (tx0, ty0).
+__device__ __forceinline__ void bt_view_setup(const ViewConst* __restrict__ vcs, int v0, int cnt, int tx0, int ty0,
+                                              BtShared& sh) {
+    for (int i = threadIdx.x; i < kBtViews; i += kBtWork) {
+        if (i >= cnt) {              // pads the last kBtUnroll views: no rays, all values 0
+            sh.vc[i] = make_int4(0, 0, 0, 0);
+            sh.a12[i] = make_float2(0.f, 0.f);
+            sh.low[i] = make_float2(__int_as_float(INT_MIN / 2), 0.f);
+            continue;
+        }
+        const ViewConst& c = vcs[v0 + i];
+        const long long qx = c.QX, qy = c.QY, h = kBtS / 2;
+        const long long qc = c.Q0 + (tx0 + h) * qx + (ty0 + h) * qy;
+        const long long ext = h * ((qx < 0 ? -qx : qx) + (qy < 0 ? -qy : qy));
+        const long long lo = ((qc - ext) >> kQFrac) - 1;      // below every pixel's q by at least one bin
+        constexpr int drop = kQFrac - kBtFrac;
+        constexpr long long half = 1ll << (drop - 1);
+        // + half a unit of the 23 bits that become the float's mantissa
+        const int base = (int)((qc - (lo << kQFrac) + half) >> drop) + (1 << (kBtFrac - 24));
+        sh.vc[i] = make_int4(base, (int)((qx + half) >> drop), (int)((qy + half) >> drop),
+                             __float_as_int(fabsf(c.a_det)));
+        const float A = fabsf(c.a_det);
+        sh.a12[i] = make_float2(1.f + A, 1.f - (A + A));
+        sh.low[i] = make_float2(__int_as_float((int)lo), c.w);
+    }
+}
+
+// Rays lo .. lo + 31 of the staged views as pairs times the path length per
+// step (0 outside the detector); true if one of them is not finite.  The
+// loads of kBtBatch views are in flight together: with a load per view and
+// trip the blocks, which all start at once, spent as long here as in the sums.
+constexpr int kBtBatch = 8;
+template <typename T>
+__device__ __forceinline__ bool bt_stage(const T* __restrict__ sino, int v0, int cnt, int nd, BtShared& sh) {
+    const int lane = threadIdx.x & 31;
+    constexpr int nw = kBtWork / 32;
+    const int pad = (cnt + kBtUnroll - 1) / kBtUnroll * kBtUnroll;
+    bool bad = false;
+    for (int i0 = threadIdx.x >> 5; i0 < pad; i0 += nw * kBtBatch) {
+        float v[kBtBatch];
+#pragma unroll
+        for (int k = 0; k < kBtBatch; ++k) {
+            const int i = min(i0 + nw * k, kBtViews - 1);
+            const float2 lw = sh.low[i];
+            const int d = __float_as_int(lw.x) + lane;
+            v[k] = 0.f;
+            if ((unsigned)d < (unsigned)nd) v[k] = ldf(sino + (size_t)(v0 + i) * nd + d) * lw.y;
+        }
+#pragma unroll
+        for (int k = 0; k < kBtBatch; ++k) {
+            const int i = i0 + nw * k;
+            const float up = __shfl_down_sync(0xffffffffu, v[k], 1);
+            bad |= !(fabsf(v[k]) <= 3.402823466e38f);
+            if (i < pad) sh.seg[i][lane] = make_float2(v[k], up);
+        }
+    }
+    return bad;
+}
+
+// Barrier of the kBtWork pixel threads alone; with a predicate, its OR over them.
+__device__ __forceinline__ void bt_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(kBtWork) : "memory"); }
+__device__ __forceinline__ bool bt_sync_or(bool p) {
+    int r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, 1, %2, p;\n\t"
+        "selp.b32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(r)
+        : "r"((int)p), "n"(kBtWork)
+        : "memory");
+    return r != 0;
+}
+
+// acc += the taps of a pixel at position q (both rays of the view).  SAFE:
+// a ray of weight 0 adds nothing even if its value is infinite or NaN.
+template <bool SAFE>
+__device__ __forceinline__ void bt_tap(const float2* __restrict__ seg, unsigned q, float A, float2 a12, float& acc) {
+    const float2 v = seg[q >> kBtFrac];
+    // 1 + fraction of q from its top 23 fraction bits
+    const float f = __uint_as_float(0x3F800000u | ((q >> (kBtFrac - 23)) & 0x7FFFFFu));
+    const float w0 = __saturatef(fmaf(-A, f, a12.x)), w1 = __saturatef(fmaf(A, f, a12.y));
+    if (!SAFE || w0 > 0.f) acc = fmaf(w0, v.x, acc);
+    if (!SAFE || w1 > 0.f) acc = fmaf(w1, v.y, acc);
+}
+
+template <bool SAFE>
+__device__ __forceinline__ void bt_views(const BtShared& sh, int cnt, int lx, int ly, float& acc0, float& acc1) {
+    for (int i0 = 0; i0 < cnt; i0 += kBtUnroll) {
+        float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < kBtUnroll; ++k) {
+            const int4 c = sh.vc[i0 + k];
+            const float2 a12 = sh.a12[i0 + k];
+            const float A = __int_as_float(c.w);
+            const unsigned q = (unsigned)c.x + (unsigned)(lx * c.y) + (unsigned)(ly * c.z);
+            bt_tap<SAFE>(sh.seg[i0 + k], q, A, a12, t0);
+            bt_tap<SAFE>(sh.seg[i0 + k], q + 8u * (unsigned)c.z, A, a12, t1);
+        }
+        acc0 += t0;
+        acc1 += t1;
+    }
+}
+
 // Tile (bx, by) of the image; `first` marks the block that records the
-// scalars (bp_tau_r) -- block (0, 0) of the slice.
+// scalars (bp_tau_r) -- block (0, 0) of the slice.  Thread t takes the pixels
+// (t % 16, t / 16) and (t % 16, t / 16 + 8) of the tile.
 template <typename T>
 __device__ __forceinline__ void backproject_tile_block(const T* __restrict__ sino, int nv, int nd, int n,
                                                        const ViewConst* __restrict__ vcs,
@@ -494,52 +585,62 @@ __device__ __forceinline__ void backproject_tile_block(const T* __restrict__ sin
                                                        int update, DevScalars* __restrict__ S,
                                                        const double* __restrict__ partial, int nparts, double M,
                                                        int bx, int by, bool first, BtShared& sh) {
-    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+    const int tid = threadIdx.x;
     const int tx0 = bx * kBtS, ty0 = by * kBtS;
-    auto& accL = sh.accL;
-    auto& accR = sh.accR;
-    auto& s_max = sh.s_max;
-    auto& s_tau_r = sh.s_tau_r;
-    float* AL = accL[wp];
-    float* AR = accR[wp];
-    for (int i = lane; i < kBtS * kBtLd; i += 32) AL[i] = AR[i] = 0.f;
-    if (tid == 0) s_max = 0u;
-    pdl_wait();      // H s and the tau_s partials are the previous kernel's output
-    if (update && wp == 0) bp_tau_r(S, partial, nparts, M, (double)n * n, &s_tau_r, first);
-    __syncwarp();
-    for (int v = wp; v < nv; v += kBtWarps) {
-        const ViewConst c = vcs[v];
-        const T* row = sino + (size_t)v * nd;
-        if (c.col)
-            bp_tile_view<1>(c, row, nd, n, tx0, ty0, AL, AR);
-        else
-            bp_tile_view<0>(c, row, nd, n, tx0, ty0, AL, AR);
-        __syncwarp();
-    }
-    __syncthreads();
-    for (int p = tid; p < kBtS * kBtS; p += blockDim.x) {
-        const int ly = p / kBtS, lx = p % kBtS;
-        const int ix = tx0 + lx, iy = ty0 + ly;
-        if (ix >= n || iy >= n) continue;
-        float t = 0.f;
+    const int lx = (tid & 15) - kBtS / 2, ly = (tid >> 4) - kBtS / 2;      // relative to pixel (8, 8)
+    const int ix = tx0 + (tid & 15), iy0 = ty0 + (tid >> 4);
+    float acc0 = 0.f, acc1 = 0.f, xi[2] = {0.f, 0.f};
+    if (tid >= kBtWork) {             // update only
+        if (tid == kBtWork) sh.s_max = 0u;
+        pdl_wait();
+        bp_tau_r(S, partial, nparts, M, (double)n * n, &sh.s_tau_r, first);
+    } else {
+        bt_view_setup(vcs, 0, min(nv, kBtViews), tx0, ty0, sh);            // plan constants: before the wait
+        pdl_wait();      // H s and the tau_s partials are the previous kernel's output
+        if (update && ix < n)
 #pragma unroll
-        for (int w = 0; w < kBtWarps; ++w) t += accL[w][ly * kBtLd + lx] + accR[w][ly * kBtLd + lx];
+            for (int h = 0; h < 2; ++h)
+                if (iy0 + 8 * h < n) xi[h] = x_in[(size_t)(iy0 + 8 * h) * n + ix];
+        for (int v0 = 0; v0 < nv; v0 += kBtViews) {
+            const int cnt = min(kBtViews, nv - v0);
+            if (v0 > 0) {
+                bt_sync();                                                 // the previous views are done with
+                bt_view_setup(vcs, v0, cnt, tx0, ty0, sh);
+            }
+            bt_sync();
+            const bool bad = bt_stage(sino, v0, cnt, nd, sh);
+            if (bt_sync_or(bad))
+                bt_views<true>(sh, cnt, lx, ly, acc0, acc1);
+            else
+                bt_views<false>(sh, cnt, lx, ly, acc0, acc1);
+        }
+    }
+    if (update) __syncthreads();      // tau_r
+    float rmax = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int iy = iy0 + 8 * h;
+        if (tid >= kBtWork || ix >= n || iy >= n) continue;
         const size_t o = (size_t)iy * n + ix;
+        const float t = h ? acc1 : acc0;
         if (update) {
-            const float rv = fmaf(s_tau_r, t, x_in[o]);
+            const float rv = fmaf(sh.s_tau_r, t, xi[h]);
             out[o] = rv;
-            atomicMax(&s_max, __float_as_uint(fabsf(rv)));
+            // |r| >= 0, so its float bit pattern orders like the value (a NaN above all)
+            rmax = __uint_as_float(max(__float_as_uint(rmax), __float_as_uint(fabsf(rv))));
         } else {
             out[o] = t;
         }
     }
     if (!update) return;
+    const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));
+    if ((tid & 31) == 0) atomicMax(&sh.s_max, wm);
     __syncthreads();
-    if (tid == 0) atomicMax(&S->rmax_bits, s_max);
+    if (tid == 0) atomicMax(&S->rmax_bits, sh.s_max);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kBtWarps * 32, 5)    // 48 registers: 5 blocks per SM, no spills
+__global__ void __launch_bounds__(kBtThreads, 8)
 k_backproject_tile(const T* __restrict__ sino, int nv, int nd, int n, const ViewConst* __restrict__ vcs,
                    const float* __restrict__ x_in, float* __restrict__ out, int update,
                    DevScalars* __restrict__ S, const double* __restrict__ partial, int nparts, double M) {
@@ -551,7 +652,7 @@ k_backproject_tile(const T* __restrict__ sino, int nv, int nd, int n, const View
 // r = x + tau_r A^T H s of every slice of a batch in one launch (after the
 // cluster sinogram kernel: one tau_s partial per view).
 template <typename T>
-__global__ void __launch_bounds__(kBtWarps * 32, 5)
+__global__ void __launch_bounds__(kBtThreads, 8)
 k_backproject_tile_batch(const BatchSlice* __restrict__ sl, const uint16_t* __restrict__ map) {
     __shared__ BtShared sh;
     const BatchSlice& B = sl[map[blockIdx.x]];
@@ -570,11 +671,12 @@ int launch_backproject(const dgamp_ct_plan_s* pl, const float* sino, const float
     if (pl->bp_mode == 1) {
         dim3 grd((pl->n + kBtS - 1) / kBtS, (pl->n + kBtS - 1) / kBtS);
         const ViewConst* vc = pl->ws.vc;
+        const dim3 blk(update ? kBtThreads : kBtWork);
         if (bf)
-            DGCT_CUDA(launch_pdl(k_backproject_tile<bf16s>, grd, dim3(kBtWarps * 32), 0, st, (const bf16s*)sino,
+            DGCT_CUDA(launch_pdl(k_backproject_tile<bf16s>, grd, blk, 0, st, (const bf16s*)sino,
                                  pl->nv, pl->nd, pl->n, vc, x_in, out, update, pl->ws.S, part, nparts, M));
         else
-            DGCT_CUDA(launch_pdl(k_backproject_tile<float>, grd, dim3(kBtWarps * 32), 0, st, sino, pl->nv, pl->nd,
+            DGCT_CUDA(launch_pdl(k_backproject_tile<float>, grd, blk, 0, st, sino, pl->nv, pl->nd,
                                  pl->n, vc, x_in, out, update, pl->ws.S, part, nparts, M));
         return DGAMP_CT_OK;
     }
@@ -607,7 +709,7 @@ int launch_project_batch(const BatchExec& E, cudaStream_t st) {
 int launch_backproject_batch(const BatchExec& E, cudaStream_t st) {
     const BatchSlice* sl = E.sl;
     const uint16_t* map = E.map[kPhBp];
-    const dim3 grd(E.nblk[kPhBp]), blk(kBtWarps * 32);
+    const dim3 grd(E.nblk[kPhBp]), blk(kBtThreads);
     if (E.bf)
         DGCT_CUDA(launch_pdl(k_backproject_tile_batch<bf16s>, grd, blk, 0, st, sl, map));
     else
