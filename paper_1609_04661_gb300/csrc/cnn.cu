@@ -225,14 +225,47 @@ __global__ void k_dgrad_last(const float* __restrict__ gout, const float* __rest
 // second kernel adds the rows in a fixed order.  Nothing depends on timing, so
 // the gradients are reproducible run to run.
 
-// grad W (reference layout [tap][ci][co]) = sum over groups of
-// partial[group][tap][ci][co] (the tensor-core kernel's layout)
-__global__ void k_reduce_wgrad64(const float* __restrict__ partial, int ngroups, float* __restrict__ gw) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;     // index in [tap][ci][co]
-    if (i >= 9 * CH * CH) return;
-    float s = 0.f;
-    for (int gq = 0; gq < ngroups; ++gq) s += partial[(size_t)gq * 9 * CH * CH + i];
-    gw[i] = s;
+// Gradients of nl hidden layers = sum over groups of partial[z][group], in the
+// weight-gradient kernel's layout ([column][lane], conv_tc.cu); layer z goes to
+// gw - z * stride (the layers run backwards), as W [tap][ci][co] then b, the
+// flat parameter order.  A thread sums four lanes of a column over every fourth
+// group, and the four threads of such a quad add by shuffles: one thread per
+// sum made the reads of a layer's rows one long chain.
+__global__ void __launch_bounds__(256) k_reduce_wgrad64(const float* __restrict__ partial, int ngroups, int width,
+                                                        float* __restrict__ gw, long long stride) {
+    const int z = blockIdx.y, i = (blockIdx.x * 256 + threadIdx.x) >> 2, part = threadIdx.x & 3;
+    const int col = i >> 5, m = (i & 31) * 4;            // column 0..383 and first lane
+    const int r = (col % 192) >> 6, co = col & 63;
+    const bool second = col >= 192, bias = second && m == 64 && r == 1;
+    const bool live = col < 384 && (!second || m < 64 || bias);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float* __restrict__ p = partial + (size_t)z * ngroups * width + (live ? col * 128 + m : 0);
+    for (int q = part; q < ngroups; q += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(p + (size_t)q * width);
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+        s.z += __shfl_xor_sync(0xffffffffu, s.z, o);
+        s.w += __shfl_xor_sync(0xffffffffu, s.w, o);
+    }
+    if (!live || part != 0) return;
+    float* g = gw - z * stride;
+    if (bias) {
+        g[9 * CH * CH + co] = s.x;
+        return;
+    }
+    const int tap = 3 * (2 - r) + (second ? 2 : m >> 6);
+    float* dst = g + (size_t)(tap * CH + (m & 63)) * CH + co;      // lanes m .. m + 3 are ci, ci + 1, ..
+    dst[0] = s.x;
+    dst[CH] = s.y;
+    dst[2 * CH] = s.z;
+    dst[3 * CH] = s.w;
 }
 
 // out[col] = sum over rows of partial[row][col]: one warp per column, the
@@ -290,22 +323,6 @@ __device__ __forceinline__ void unpack8(const uint4& v, float* f) {
         f[2 * k] = t.x;
         f[2 * k + 1] = t.y;
     }
-}
-
-// bias gradient: partial[block][c] = sum over the block's pixels of g[p][c]
-__global__ void __launch_bounds__(256) k_bias_partial(const bf16* __restrict__ g, long long npix, long long per,
-                                                      float* __restrict__ partial) {
-    __shared__ float sm[8][CH];
-    const int cg = threadIdx.x & 7, pl = threadIdx.x >> 3;
-    const long long p0 = (long long)blockIdx.x * per, p1 = std::min(p0 + per, npix);
-    float s[1][8] = {};
-    for (long long p = p0 + pl; p < p1; p += 32) {
-        float f[8];
-        unpack8(*reinterpret_cast<const uint4*>(g + p * CH + cg * 8), f);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) s[0][k] += f[k];
-    }
-    block_colsum<1>(s, sm, partial + (size_t)blockIdx.x * CH);
 }
 
 // First layer: partial[block][tap*64 + co] = sum_p u[p + off(tap)] g1[p][co];
@@ -455,8 +472,8 @@ struct dgamp_ct_cnn_s {
     int64_t cap_pix = 0;
     int cap_store = 0;    // activations kept for all layers (training), 2 (inference) or 4 (with tangent)
     bf16* act = nullptr;  // [cap_store][cap_pix][64]
-    bf16* g0 = nullptr;   // [cap_pix][64]
-    bf16* g1 = nullptr;
+    bf16* g = nullptr;    // [n_g][cap_pix][64] output gradients of consecutive layers (training)
+    int n_g = 0;
     float* f = nullptr;   // [cap_pix]
     float* gout = nullptr;
     float* partial = nullptr;   // wgrad partials
@@ -470,13 +487,15 @@ struct dgamp_ct_cnn_s {
     uint64_t ws_gen = 0;        // bumped whenever the workspace is reallocated or captured launches change
 };
 
-constexpr int kWgGroupsMax = 64;   // most CTA groups of the tensor-core weight gradient
+constexpr int kWgGroupsMax = 64;            // most CTA groups of the tensor-core weight gradient
+constexpr size_t kGradBytes = 1ull << 30;   // bound on the gradients kept for it
 
 static void cnn_free_ws(dgamp_ct_cnn_s* c) {
-    void* ptrs[] = {c->act, c->g0, c->g1, c->f, c->gout, c->partial, c->dpart, c->loss, c->sig_buf};
+    void* ptrs[] = {c->act, c->g, c->f, c->gout, c->partial, c->dpart, c->loss, c->sig_buf};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    c->act = c->g0 = c->g1 = nullptr;
+    c->act = c->g = nullptr;
+    c->n_g = 0;
     c->f = c->gout = c->partial = c->sig_buf = nullptr;
     c->dpart = c->loss = nullptr;
     c->cap_pix = 0;
@@ -497,12 +516,19 @@ static int cnn_ensure_ws(dgamp_ct_cnn_s* c, int64_t npix, int nstore, int batch)
     };
     int rc;
     if ((rc = A((void**)&c->act, (size_t)ns * cap * CH * sizeof(bf16))) != DGAMP_CT_OK) return rc;
-    if ((rc = A((void**)&c->g0, (size_t)cap * CH * sizeof(bf16))) != DGAMP_CT_OK) return rc;
-    if ((rc = A((void**)&c->g1, (size_t)cap * CH * sizeof(bf16))) != DGAMP_CT_OK) return rc;
+    // gradients of all layers where they fit kGradBytes, so that one launch takes every layer's
+    // weight gradient; else of as many as fit, and of two at least (as much as a layer by layer pass needs)
+    const size_t slot = (size_t)cap * CH * sizeof(bf16);
+    if (ns >= c->L - 1) {   // training
+        c->n_g = (int)std::min<size_t>(c->L - 1, std::max<size_t>(2, kGradBytes / slot));
+        if ((rc = A((void**)&c->g, c->n_g * slot)) == DGAMP_CT_ERR_OOM) rc = A((void**)&c->g, (c->n_g = 2) * slot);
+        if (rc != DGAMP_CT_OK) return rc;
+    }
     if ((rc = A((void**)&c->f, (size_t)cap * sizeof(float))) != DGAMP_CT_OK) return rc;
     if ((rc = A((void**)&c->gout, (size_t)cap * sizeof(float))) != DGAMP_CT_OK) return rc;
     // the larger of the tensor-core weight gradient's partials and the pixel sums' (+ their reduction)
-    const size_t n_part = std::max((size_t)kWgGroupsMax * 9 * CH * CH, (size_t)(kColBlocks + 1) * 10 * CH);
+    const size_t n_part = std::max((size_t)std::max(c->sm_count, kWgGroupsMax) * wgrad64_partial_floats(),
+                                   (size_t)(kColBlocks + 1) * 10 * CH);
     if ((rc = A((void**)&c->partial, n_part * sizeof(float))) != DGAMP_CT_OK) return rc;
     if ((rc = A((void**)&c->dpart, 1024 * sizeof(double))) != DGAMP_CT_OK) return rc;
     if ((rc = A((void**)&c->loss, sizeof(double))) != DGAMP_CT_OK) return rc;
@@ -555,9 +581,6 @@ static int cnn_backward(dgamp_ct_cnn_s* c, const float* r, const float* sig, int
     const int nb = col_blocks(npix);
     const long long per = (npix + nb - 1) / nb;
     const unsigned rgrid = (unsigned)((10 * CH + 7) / 8);   // k_reduce_cols: 8 columns per 256 threads
-    // CTA groups of the hidden layers' weight gradient: 3 CTAs (one per tap
-    // row) per group, about one CTA per SM
-    const int Gw = std::max(1, std::min(kWgGroupsMax, c->sm_count / 3));
     // last layer weights and bias
     k_wgrad_last<<<nb, 256, 0, st>>>(act(L - 1), c->gout, B, H, W, per, c->partial);
     DGCT_LAUNCH_CHECK();
@@ -567,25 +590,28 @@ static int cnn_backward(dgamp_ct_cnn_s* c, const float* r, const float* sig, int
     // scatter [tap*64+ci] -> grad W[L-1] ([tap][ci][1]) and [9*64] -> b
     DGCT_CUDA(cudaMemcpyAsync(c->grad + c->w_off[L - 1], red, 9 * CH * sizeof(float), cudaMemcpyDeviceToDevice, st));
     DGCT_CUDA(cudaMemcpyAsync(c->grad + c->b_off[L - 1], red + 9 * CH, sizeof(float), cudaMemcpyDeviceToDevice, st));
-    bf16* gcur = c->g0;
-    bf16* gnext = c->g1;
-    k_dgrad_last<<<blocks, 128, 0, st>>>(c->gout, c->w16, act(L - 1), gcur, B, H, W);
+    auto grad = [&](int k) -> bf16* { return c->g + (size_t)k * c->cap_pix * CH; };
+    int at = 0, dir = 1;   // slot of the current layer's output gradient; the slots fill upwards, then back down
+    k_dgrad_last<<<blocks, 128, 0, st>>>(c->gout, c->w16, act(L - 1), grad(0), B, H, W);
     DGCT_LAUNCH_CHECK();
-    for (int l = L - 2; l >= 1; --l) {
-        // layer l maps a_l -> z_{l+1}; gcur = dL/dz_{l+1}
-        DGCT_TRY(launch_wgrad64_tc(act(l), gcur, B, H, W, Gw, c->partial, c->tc_err, st, c->stall_ns));
-        k_reduce_wgrad64<<<(9 * CH * CH + 255) / 256, 256, 0, st>>>(c->partial, Gw, c->grad + c->w_off[l]);
+    const int width = wgrad64_partial_floats();
+    for (int l = L - 2; l >= 1;) {
+        // layer l maps a_l -> z_{l+1}; slot `at` holds dL/dz_{l+1}.  The input gradients of nl layers,
+        // then their weight and bias gradients in one launch, about one CTA per SM
+        const int nl = std::min(l, c->n_g - 1), first = at;
+        for (int z = 0; z < nl; ++z, at += dir)
+            DGCT_TRY(launch_conv64_tc(1, grad(at), c->wt, L - 2, l - z - 1, nullptr, act(l - z), grad(at + dir), B, H,
+                                      W, c->sm_count, c->tc_err, st, c->stall_ns));
+        const int Gw = std::max(1, std::min(kWgGroupsMax, c->sm_count / nl));
+        DGCT_TRY(launch_wgrad64_tc(c->act, c->cap_store, l - 1, c->g, c->n_g, first, dir, c->cap_pix, nl, B, H, W, Gw,
+                                   c->partial, c->tc_err, st, c->stall_ns));
+        k_reduce_wgrad64<<<dim3((width + 255) / 256, nl), 256, 0, st>>>(c->partial, Gw, width, c->grad + c->w_off[l],
+                                                                       9LL * CH * CH + CH);
         DGCT_LAUNCH_CHECK();
-        k_bias_partial<<<nb, 256, 0, st>>>(gcur, npix, per, c->partial);
-        DGCT_LAUNCH_CHECK();
-        k_reduce_cols<<<(CH + 7) / 8, 256, 0, st>>>(c->partial, nb, CH, c->grad + c->b_off[l]);
-        DGCT_LAUNCH_CHECK();
-        DGCT_TRY(launch_conv64_tc(1, gcur, c->wt, L - 2, l - 1, nullptr, act(l), gnext, B, H, W, c->sm_count,
-                                  c->tc_err, st, c->stall_ns));
-        bf16* t = gcur;
-        gcur = gnext;
-        gnext = t;
+        l -= nl;
+        dir = -dir;
     }
+    bf16* gcur = grad(at);
     // first layer: gcur = dL/dz_1
     k_wgrad_first<<<nb, 256, 0, st>>>(r, sig, gcur, B, H, W, per, c->partial);
     DGCT_LAUNCH_CHECK();

@@ -192,19 +192,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
         : "r"(taddr));
 }
 
-// 16 consecutive FP32 accumulator columns of this warp's 32 TMEM lanes
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 typedef __nv_bfloat16 bf16;
 
 // Strip s of the batch (row fastest): band = s / H is a 128-column band of
@@ -497,68 +484,90 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
 }
 
 // ---------------------------------------------------- weight gradient ----
-// partial[group][tap][ci][co] = sum over the group's pixels p of
-//   g[p][co] a[p + (dy - 1, dx - 1)][ci],   tap = 3 dy + dx,
-// a GEMM per tap with M = 64 output channels, N = 64 input channels and the
-// pixels as K.  Both operands lie pixel-major in global memory (one pixel's
-// 64 channels = one 128-byte row), which read with pixels as K is the
-// MN-major operand layout with the 128-byte swizzle: the same TMA copies as
-// the forward kernel's (a strip of 128 gradient pixels, a halo row of 130
-// activation pixels) feed the MMAs with no transposition, and the three dx
-// taps of a row start 0, 1 and 2 pixel rows into the halo row.
+// For a layer with input activations a and output gradient g,
+//   partial[tap][ci][co] = sum over pixels p of a[p + (dy - 1, dx - 1)][ci] g[p][co],  tap = 3 dy + dx,
+// and the bias gradient sum_p g[p][co]: GEMMs with the pixels as K.  Both
+// operands lie pixel-major in global memory (one pixel's 64 channels = one
+// 128-byte row), which read with pixels as K is the MN-major operand layout
+// with the 128-byte swizzle, so the convolution's TMA copies (a halo row of
+// 130 activation pixels, a strip of 128 gradient pixels) feed the MMAs as they
+// land.
 //
-// CTA (group, dy) takes a contiguous range of strips and accumulates taps
-// (dy, 0..2) over all of them in tensor memory: three 64-column FP32
-// accumulators.  With M = 64 the accumulator's row m lies in TMEM lane
-// 32 (m / 16) + m % 16 (the first 16 lanes of each quarter); the four
-// warps read their quarters once, at the end.  Warp 0 (one lane) loads
-// strips into a ring of WG_STAGES stages, warp 1 (one lane) issues 3 x 8
-// MMAs per strip and releases the stage with a commit.
-constexpr int WG_G_BYTES = M * 128;                    // 128 gradient pixels
-constexpr int WG_STAGE = WG_G_BYTES + A_ROW;           // + one halo row slot (136 pixels)
-constexpr int WG_STAGES = 5;
-constexpr int WG_SMEM = 1024 + WG_STAGES * WG_STAGE;
-constexpr int WG_THREADS = 128;
-constexpr unsigned WG_TMEM_COLS = 256;                 // three 64-column accumulators
-// kind::f16 instruction descriptor: D FP32, A and B BF16, both MN-major, N = 64, M = 64
-constexpr uint32_t IDESC_WG = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                              ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(64 >> 4) << 24);
+// All nine taps and the bias of an activation row take two MMAs per 16 pixels,
+// both M = 128, N = 192:
+//   B = the gradient rows above, at and below the activation row (N = 3 x 64,
+//       one row slot apart; they are its dy = 2, 1 and 0 taps);
+//   A = the activation row twice, the second copy starting one pixel later
+//       (M = 2 x 64, the leading-dimension offset is one 128-byte row): dx = 0
+//       and 1; then once more from pixel 2, beside a block of ones: dx = 2 and,
+//       in the ones' rows, the gradient's own sums.
+// M = 64 halves fill half of the tensor core, and separate CTAs per dy read
+// both operands three times: that form took 25.5 us per layer on 32 patches of
+// 64 x 64 and two more kernels for the bias; this one takes
+// 12 us per layer (ncu; the whole training pass 1296 -> 891 us).
+//
+// One launch covers several layers (blockIdx.y): each CTA sums its layer over a
+// contiguous range of strips.  The tensor core truncates as it accumulates, an
+// error that grows with the number of additions, so after at most WG_CHAIN
+// steps of 16 pixels the sums move from tensor memory to the CTA's partial,
+// where one thread per element adds them up in FP32 (1e-5 relative without, at
+// 816 steps).  Warp 0 (one lane) loads rows, warp 1 issues the MMAs, warps 4..7
+// move the sums; gradient rows pass through a ring, and where three of them
+// wrap around its end the MMA is split in two.
+constexpr int WG_G_SLOT = M * 128;                     // 128 gradient pixels
+constexpr int WG_NA = 4, WG_NG = 6;                    // row slots of the two rings
+constexpr int WG_ONES = 2048;                          // 16 pixels x 64 ones
+constexpr int WG_SMEM = 1024 + WG_NA * A_ROW + WG_NG * WG_G_SLOT + WG_ONES;
+constexpr int WG_THREADS = 256;
+constexpr int WG_CHAIN = 320;                          // most accumulation steps (a row may start below, and end past it)
+constexpr unsigned WG_TMEM_COLS = 512;                 // two 192-column accumulators (a power of two)
+// One partial as it lies in tensor memory, [column][lane], so that a warp's lanes write whole lines.  Column
+// 64 r + co of the first accumulator: tap dy = 2 - r, dx = lane / 64, ci = lane % 64; of the second: lanes below 64
+// dx = 2, lane 64 of r = 1 the bias, the others nothing.
+constexpr int WG_OUT = 2 * 192 * 128;
+// kind::f16 instruction descriptor: D FP32, A and B BF16, both MN-major, M = 128, N = 64 count
+__device__ __forceinline__ uint32_t idesc_wg(int count) { return idesc_n(count) | (1u << 15) | (1u << 16); }
 
-// MN-major operand, 128-byte swizzle, 64 elements along M or N (one swizzle
-// atom, so the leading-dimension offset is not used): rows of 128 bytes are
-// successive K (pixels), 8-row groups 1024 bytes apart.  The swizzle follows
-// the absolute shared-memory address, as the TMA wrote it, so the start may
-// move by whole rows.
-__device__ __forceinline__ uint64_t sdesc_sw128_mn(uint32_t saddr) {
-    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)1u << 16) | ((uint64_t)(1024u >> 4) << 32) |
-           (1ull << 46) | (2ull << 61);
+// accumulation steps of strip s (past the image the gradient is 0)
+__device__ __forceinline__ int wg_steps(int s, int H, int W, int nx) {
+    const int wide = W - strip_of(s, H, nx).x0;
+    return ((wide < M ? wide : M) + 15) / 16;
+}
+
+// MN-major operand, 128-byte swizzle: 64 elements along M or N per 128-byte
+// row, rows are successive K (pixels), 8-row groups 1024 bytes apart, the next
+// 64 elements along M or N `lbo` bytes on.  The swizzle follows the absolute
+// shared-memory address, as the TMA wrote it, so a start may move by whole rows.
+__device__ __forceinline__ uint64_t sdesc_sw128_mn(uint32_t saddr, uint32_t lbo) {
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
+           ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
 __global__ void __launch_bounds__(WG_THREADS, 1)
-k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_g, int B, int H,
-             int W, int per, float* __restrict__ partial, unsigned* err, unsigned long long stall_ns) {
+k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_g, int a_first,
+             int g_first, int g_step, int B, int H, int W, int per, float* __restrict__ partial, unsigned* err,
+             unsigned long long stall_ns) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full[WG_STAGES];
-    __shared__ __align__(8) uint64_t empty[WG_STAGES];
-    __shared__ __align__(8) uint64_t acc_full;
+    __shared__ __align__(8) uint64_t a_full[WG_NA], a_empty[WG_NA], g_full[WG_NG], g_empty[WG_NG];
+    __shared__ __align__(8) uint64_t acc_full, acc_empty;
     __shared__ __align__(8) uint64_t never_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int stalled;
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
-    const int group = blockIdx.x, dy = blockIdx.y;
+    const int group = blockIdx.x, z = blockIdx.y;
+    const int la = a_first - z, lg = g_first + g_step * z;    // layer slots of the two tensors
     const uint32_t raw = smem_u32(smem_raw);
-    const uint32_t s_base = (raw + 1023u) & ~1023u;
+    const uint32_t sA = (raw + 1023u) & ~1023u, sG = sA + WG_NA * A_ROW, sOnes = sG + WG_NG * WG_G_SLOT;
     const int nx = (W + M - 1) / M;
     const int nstrips = B * H * nx;
     const int s0 = group * per;
     const int s1 = s0 + per < nstrips ? s0 + per : nstrips;
-    float* out = partial + ((size_t)group * 9 + 3 * dy) * CH * CH;
+    float* out = partial + ((size_t)z * gridDim.x + group) * WG_OUT;
     if (s0 >= s1) {   // no strips: zero partials
-        for (int i = tid; i < 3 * CH * CH; i += WG_THREADS) out[i] = 0.f;
+        for (int i = tid; i < WG_OUT; i += WG_THREADS) out[i] = 0.f;
         return;
     }
-    const int nk = s1 - s0;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_slot)),
                      "r"(WG_TMEM_COLS)
@@ -566,15 +575,23 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     if (tid == 0) {
-        for (int s = 0; s < WG_STAGES; ++s) {
-            mbar_init(smem_u32(&full[s]), 1);
-            mbar_init(smem_u32(&empty[s]), 1);
+        for (int s = 0; s < WG_NA; ++s) {
+            mbar_init(smem_u32(&a_full[s]), 1);
+            mbar_init(smem_u32(&a_empty[s]), 1);
+        }
+        for (int s = 0; s < WG_NG; ++s) {
+            mbar_init(smem_u32(&g_full[s]), 1);
+            mbar_init(smem_u32(&g_empty[s]), 1);
         }
         mbar_init(smem_u32(&acc_full), 1);
+        mbar_init(smem_u32(&acc_empty), 4);
         mbar_init(smem_u32(&never_bar), 1);
         stalled = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    for (int i = tid; i < WG_ONES / 4; i += WG_THREADS)      // BF16 1.0 pairs
+        asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(sOnes + 4 * i), "r"(0x3F803F80u) : "memory");
+    fence_async_smem();
     fence_before();
     __syncthreads();
     fence_after();
@@ -587,74 +604,125 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     }
     bool ok = run;
     if (run && warp == 0 && lane == 0) {
-        // ---- TMA producer ----
-        int k = 0;
-        for (; k < nk; ++k) {
-            const int st = k % WG_STAGES;
-            if (k >= WG_STAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((k / WG_STAGES - 1) & 1))) {
-                ok = false;
-                break;
-            }
-            const Strip t = strip_of(s0 + k, H, nx);
-            const uint32_t sg = s_base + (uint32_t)(st * WG_STAGE), sa = sg + WG_G_BYTES;
-            const uint32_t bar = smem_u32(&full[st]);
-            mbar_expect_tx(bar, WG_G_BYTES + ROW_BYTES);
-            tma_4d(sg, &map_g, 0, t.x0, t.y, t.b, bar);
-            tma_4d(sa, &map_a, 0, t.x0 - 1, t.y + dy - 1, t.b, bar);
+        // ---- TMA producer: per run of activation rows y .. y + R - 1 of a band, gradient rows y - 1 .. y + R ----
+        int qa = 0, qg = 0;
+        auto put = [&](bool act, const Strip& t, int y) {
+            int& q = act ? qa : qg;
+            const int n = act ? WG_NA : WG_NG, slot = q % n;
+            uint64_t* full = act ? a_full : g_full;
+            uint64_t* empty = act ? a_empty : g_empty;
+            if (q >= n && !mbar_wait(smem_u32(&empty[slot]), (uint32_t)((q / n - 1) & 1))) return false;
+            const uint32_t bar = smem_u32(&full[slot]);
+            mbar_expect_tx(bar, act ? ROW_BYTES : WG_G_SLOT);
+            if (act)
+                tma_5d(sA + (uint32_t)(slot * A_ROW), &map_a, 0, t.x0 - 1, y, t.b, la, bar);
+            else
+                tma_5d(sG + (uint32_t)(slot * WG_G_SLOT), &map_g, 0, t.x0, y, t.b, lg, bar);
+            ++q;
+            return true;
+        };
+        for (int s_a = s0; ok && s_a < s1;) {
+            const int s_e = run_end(s_a, s1, H);
+            const Strip t = strip_of(s_a, H, nx);
+            ok = put(false, t, t.y - 1) && put(false, t, t.y);
+            for (int i = 0; ok && i <= s_e - s_a; ++i) ok = put(false, t, t.y + i + 1) && put(true, t, t.y + i);
+            s_a = s_e + 1;
         }
         // every copy issued has landed before the CTA may exit (bounded)
-        for (int j = (k > WG_STAGES ? k - WG_STAGES : 0); j < k; ++j)
-            if (!mbar_wait(smem_u32(&full[j % WG_STAGES]), (uint32_t)((j / WG_STAGES) & 1))) ok = false;
+        for (int j = qa > WG_NA ? qa - WG_NA : 0; j < qa; ++j)
+            if (!mbar_wait(smem_u32(&a_full[j % WG_NA]), (uint32_t)((j / WG_NA) & 1))) ok = false;
+        for (int j = qg > WG_NG ? qg - WG_NG : 0; j < qg; ++j)
+            if (!mbar_wait(smem_u32(&g_full[j % WG_NG]), (uint32_t)((j / WG_NG) & 1))) ok = false;
     } else if (run && warp == 1) {
         // ---- MMA issuer (the whole warp, one elected lane issues) ----
-        for (int k = 0; k < nk; ++k) {
-            const int st = k % WG_STAGES;
-            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[st]), (uint32_t)((k / WG_STAGES) & 1)))) {
-                ok = false;
-                break;
-            }
-            fence_after();
-            const uint32_t sg = s_base + (uint32_t)(st * WG_STAGE), sa = sg + WG_G_BYTES;
-            const uint64_t gd = sdesc_sw128_mn(sg), ad = sdesc_sw128_mn(sa);
-#pragma unroll
-            for (int ks = 0; ks < M / 16; ++ks) {
-#pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    // 16 pixels (rows) per MMA; tap dx reads the halo row dx rows later
-                    mma_bf16(tmem + (uint32_t)(dx * 64), gd + (uint64_t)((ks * 16 * 128) >> 4),
-                             ad + (uint64_t)(((ks * 16 + dx) * 128) >> 4), IDESC_WG, (k | ks) != 0 ? 1u : 0u);
+        int qa = 0, qg = 0, seen = 0;   // activation row, first of its gradient rows, gradient rows waited for
+        int chain = 0, flushes = 0;     // steps since the accumulators were emptied, and how often they were
+        for (int s_a = s0; ok && s_a < s1;) {
+            const int s_e = run_end(s_a, s1, H);
+            const int nks = wg_steps(s_a, H, W, nx);
+            for (int i = 0; i <= s_e - s_a; ++i, ++qa, ++qg) {
+                bool got = true;
+                if (chain >= WG_CHAIN) {
+                    mma_commit(smem_u32(&acc_full));
+                    got = mbar_wait(smem_u32(&acc_empty), (uint32_t)(flushes & 1));
+                    ++flushes;
+                    chain = 0;
                 }
+                got = mbar_wait(smem_u32(&a_full[qa % WG_NA]), (uint32_t)((qa / WG_NA) & 1)) && got;
+                for (; seen < qg + 3; ++seen)
+                    got = mbar_wait(smem_u32(&g_full[seen % WG_NG]), (uint32_t)((seen / WG_NG) & 1)) && got;
+                if (!__all_sync(0xffffffffu, got)) {
+                    ok = false;
+                    break;
+                }
+                fence_after();
+                const uint32_t a0 = sA + (uint32_t)((qa % WG_NA) * A_ROW);
+                const int gs = qg % WG_NG, n1 = gs + 3 > WG_NG ? WG_NG - gs : 3, n2 = 3 - n1;
+                const uint64_t g1 = sdesc_sw128_mn(sG + (uint32_t)(gs * WG_G_SLOT), WG_G_SLOT);
+                const uint64_t g2 = sdesc_sw128_mn(sG, WG_G_SLOT);
+                const uint32_t d2 = tmem + (uint32_t)(n1 * 64), i1 = idesc_wg(n1), i2 = idesc_wg(n2);
+#pragma unroll 1
+                for (int ks = 0; ks < nks; ++ks) {
+                    const uint32_t acc = (chain | ks) != 0 ? 1u : 0u;
+                    const uint64_t go = (uint64_t)((ks * 16 * 128) >> 4);
+                    const uint32_t at = a0 + (uint32_t)(ks * 16 * 128);
+                    const uint64_t a01 = sdesc_sw128_mn(at, 128u), a2 = sdesc_sw128_mn(at + 256u, sOnes - at - 256u);
+                    mma_bf16(tmem, a01, g1 + go, i1, acc);
+                    if (n2) mma_bf16(d2, a01, g2 + go, i2, acc);
+                    mma_bf16(tmem + 192u, a2, g1 + go, i1, acc);
+                    if (n2) mma_bf16(d2 + 192u, a2, g2 + go, i2, acc);
+                }
+                chain += nks;
+                mma_commit(smem_u32(&a_empty[qa % WG_NA]));
+                mma_commit(smem_u32(&g_empty[qg % WG_NG]));
             }
-            mma_commit(smem_u32(&empty[st]));
+            if (ok)   // the run's last two gradient rows
+                for (int k = 0; k < 2; ++k, ++qg) mma_commit(smem_u32(&g_empty[qg % WG_NG]));
+            s_a = s_e + 1;
         }
         // arrives once every MMA issued above has completed
         mma_commit(smem_u32(&acc_full));
-    }
-    __syncwarp();
-    // ---- epilogue: all four warps, once ----
-    if (run) {
-        int got = 0;
-        if (lane == 0) got = mbar_wait(smem_u32(&acc_full), 0u) ? 1 : 0;
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (!got) {
-            ok = false;
-        } else {
+    } else if (run && warp >= 4) {
+        // ---- sums from tensor memory to the partial: stored the first time, then added (each element by
+        // one thread, so in a fixed order) ----
+        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+        const int m = (warp & 3) * 32 + lane;
+        int chain = 0, flushes = 0;
+        for (int s = s0; s < s1; ++s) {
+            chain += wg_steps(s, H, W, nx);
+            if (chain < WG_CHAIN && s + 1 < s1) continue;
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full), (uint32_t)(flushes & 1)))) {
+                ok = false;
+                break;
+            }
             fence_after();
-            const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-            const int co = warp * 16 + lane;     // lanes 0..15 hold rows 16 warp .. + 15
 #pragma unroll 1
-            for (int c = 0; c < 3 * 64; c += 16) {
-                float v[16];
-                tmem_ld16(tmem + lane_base + (uint32_t)c, v);   // warp-collective
-                if (lane < 16) {   // 16 output channels of one warp: 64 contiguous bytes per ci
-                    const int tap = c >> 6, ci = c & 63;
-                    float* dst = out + ((size_t)tap * CH + ci) * CH + co;
+            for (int c = 0; c < 12; ++c) {   // 32 columns: accumulator c / 6, gradient row c / 2 % 3, half of co
+                uint32_t v[32];
+                __syncwarp();
+                tmem_ld32(tmem + lane_base + (uint32_t)(c * 32), v);   // warp-collective
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                if (c >= 6 && m >= 64 && !(m == 64 && (c == 8 || c == 9))) continue;
+                float* dst = out + c * 32 * 128 + m;
+                if (flushes == 0) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) dst[(size_t)j * CH] = v[j];
+                    for (int j = 0; j < 32; ++j) dst[j * 128] = __uint_as_float(v[j]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        asm volatile("red.global.add.f32 [%0], %1;\n" ::"l"(dst + j * 128), "f"(__uint_as_float(v[j]))
+                                     : "memory");
                 }
             }
+            fence_before();               // the reads are complete: the accumulators may be overwritten
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&acc_empty)) : "memory");
+            ++flushes;
+            chain = 0;
         }
     }
+    __syncwarp();
     if (!ok && (run || tid == 0)) atomicOr(err, 1u);
     fence_before();
     __syncthreads();
@@ -740,31 +808,36 @@ int launch_conv64_tc(int mode, const void* in, const void* wk_all, int layers, i
     return DGAMP_CT_OK;
 }
 
-// a: the layer's input activations, g: the gradient at its output, both
-// [B][H][W][64] BF16; partial: [groups][9][64 ci][64 co] FP32, every group
-// written (zeros for a group without strips).
-int launch_wgrad64_tc(const void* a, const void* g, int B, int H, int W, int groups, float* partial, unsigned* err,
-                      cudaStream_t st, unsigned long long stall_ns) {
-    if (groups < 1) return DGAMP_CT_ERR_INVALID_ARG;
+// Layers z = 0 .. nl - 1: input activations in slot a_first - z of `acts`,
+// output gradients in slot g_first + g_step z of `grads`, both
+// [slots][slot][64] BF16 with slot = slot_pix pixels of which the first B H W
+// are used; partial: [nl][groups][9 * 64 * 64 + 64] FP32, every one written
+// (zeros for a group without strips).
+int wgrad64_partial_floats() { return tc::WG_OUT; }
+int launch_wgrad64_tc(const void* acts, int act_slots, int a_first, const void* grads, int grad_slots, int g_first,
+                      int g_step, long long slot_pix, int nl, int B, int H, int W, int groups, float* partial,
+                      unsigned* err, cudaStream_t st, unsigned long long stall_ns) {
+    if (groups < 1 || nl < 1) return DGAMP_CT_ERR_INVALID_ARG;
     const long long nstrips = (long long)B * H * ((W + tc::M - 1) / tc::M);
     if (nstrips <= 0) {
-        DGCT_CUDA(cudaMemsetAsync(partial, 0, (size_t)groups * 9 * 64 * 64 * sizeof(float), st));
+        DGCT_CUDA(cudaMemsetAsync(partial, 0, (size_t)nl * groups * tc::WG_OUT * sizeof(float), st));
         return DGAMP_CT_OK;
     }
     CUtensorMap map_a, map_g;
-    const cuuint64_t dims[4] = {64, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
-    const cuuint64_t strides[3] = {128, (cuuint64_t)W * 128, (cuuint64_t)H * W * 128};
+    const cuuint64_t strides[4] = {128, (cuuint64_t)W * 128, (cuuint64_t)H * W * 128, (cuuint64_t)slot_pix * 128};
     {
-        const cuuint32_t box[4] = {64, (cuuint32_t)tc::HWL, 1, 1};
-        DGCT_TRY(encode(&map_a, 4, a, dims, strides, box));
+        const cuuint64_t dims[5] = {64, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B, (cuuint64_t)act_slots};
+        const cuuint32_t box[5] = {64, (cuuint32_t)tc::HWL, 1, 1, 1};
+        DGCT_TRY(encode(&map_a, 5, acts, dims, strides, box));
     }
     {
-        const cuuint32_t box[4] = {64, (cuuint32_t)tc::M, 1, 1};
-        DGCT_TRY(encode(&map_g, 4, g, dims, strides, box));
+        const cuuint64_t dims[5] = {64, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B, (cuuint64_t)grad_slots};
+        const cuuint32_t box[5] = {64, (cuuint32_t)tc::M, 1, 1, 1};
+        DGCT_TRY(encode(&map_g, 5, grads, dims, strides, box));
     }
     const int per = (int)((nstrips + groups - 1) / groups);
-    tc::k_wgrad64_tc<<<dim3(groups, 3), tc::WG_THREADS, tc::WG_SMEM, st>>>(map_a, map_g, B, H, W, per, partial, err,
-                                                                          stall_ns);
+    tc::k_wgrad64_tc<<<dim3(groups, nl), tc::WG_THREADS, tc::WG_SMEM, st>>>(map_a, map_g, a_first, g_first, g_step, B, H,
+                                                                           W, per, partial, err, stall_ns);
     DGCT_LAUNCH_CHECK();
     return DGAMP_CT_OK;
 }
