@@ -49,11 +49,13 @@ constexpr int HWL = M + 2;                // halo pixels loaded per row
 constexpr int HWP = 136;                  // row slot: 136 pixels x 128 B = 17 x 1024 B
 constexpr int A_ROW = HWP * 128;          // bytes of one row slot (pixel-major, 128-byte swizzle)
 constexpr int RING = 6;                   // row slots: one being multiplied, the others landing
+constexpr int FOLD_RING = 2;              // FOLD: slots of three shifted rows (the loads of one overlap the MMAs of the other)
 constexpr int A_BYTES = RING * A_ROW;     // the ring
 constexpr int ROW_BYTES = HWL * 128;      // bytes one row load delivers (130 pixels x 64 channels)
 constexpr int B_TAP = 64 * 128;           // one tap of the weights: 64 co x 64 ci, 128-byte swizzle
 constexpr int B_BYTES = 9 * B_TAP;        // [dx][dy][co][ci]
 constexpr int O_BYTES = M * 128;          // one strip on its way out (and its mask on the way in)
+static_assert(FOLD_RING * 3 * O_BYTES <= A_BYTES, "the shifted rows use the ring's memory");
 constexpr int EPI_GROUPS = 2;             // epilogue groups of four warps: group g drains strips k % 2 == g
 constexpr int SMEM = 1024 + B_BYTES + A_BYTES + EPI_GROUPS * O_BYTES;   // + alignment slack
 constexpr int EPI_WARP0 = 4;              // warps 4..11: epilogue; warp 0: TMA; warp 1: MMA
@@ -260,7 +262,13 @@ __device__ __forceinline__ uint32_t finish2(uint32_t r0, uint32_t r1, float2 b, 
 //     one TMA store.  The mask of the group's next strip is loaded into the
 //     same buffer once the store has read it: each lane overwrites just the
 //     mask chunk it has read.
-template <int MODE>
+//
+// FOLD (images at most 64 pixels wide, the training patches): a strip is the
+// same row of two images, 2 x 64 pixels, where a strip of one row would
+// multiply 64 pixels of padding.  The halo columns of the two rows cannot share
+// one buffer, so each row is loaded once per dx, already shifted; a slot holds
+// the three copies.
+template <int MODE, bool FOLD>
 __global__ void __launch_bounds__(THREADS, 1)
 k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_w,
             const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_mask, int layer,
@@ -281,8 +289,11 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t sB = (raw + 1023u) & ~1023u, sA = sB + B_BYTES, sO = sA + A_BYTES;
+    constexpr int ring = FOLD ? FOLD_RING : RING;
+    constexpr uint32_t slot_bytes = FOLD ? 3 * O_BYTES : A_ROW, dx_bytes = FOLD ? O_BYTES : 128;
+    constexpr int ib = FOLD ? 2 : 1;      // images per strip
     const int nx = (W + M - 1) / M;
-    const int nstrips = B * H * nx;
+    const int nstrips = (B + ib - 1) / ib * H * nx;
     const int s0 = (int)blockIdx.x * per;
     const int s1 = s0 + per < nstrips ? s0 + per : nstrips;
     if (s0 >= s1) return;
@@ -332,11 +343,18 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
                 const int s_e = run_end(s_a, s1, H);
                 const Strip t = strip_of(s_a, H, nx);
                 for (int i = 0; i < s_e - s_a + 3; ++i, ++q) {
-                    const int slot = q % RING;
-                    if (q >= RING && !mbar_wait(smem_u32(&row_empty[slot]), (uint32_t)((q / RING - 1) & 1))) ok = false;
+                    const int slot = q % ring;
+                    if (q >= ring && !mbar_wait(smem_u32(&row_empty[slot]), (uint32_t)((q / ring - 1) & 1))) ok = false;
                     const uint32_t bar = smem_u32(&row_full[slot]);
-                    mbar_expect_tx(bar, ROW_BYTES);
-                    tma_4d(sA + (uint32_t)(slot * A_ROW), &map_in, 0, t.x0 - 1, t.y - 1 + i, t.b, bar);
+                    const uint32_t dst = sA + (uint32_t)slot * slot_bytes;
+                    mbar_expect_tx(bar, FOLD ? 3 * O_BYTES : ROW_BYTES);
+                    if (FOLD) {
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx)
+                            tma_4d(dst + dx * dx_bytes, &map_in, 0, dx - 1, t.y - 1 + i, ib * t.b, bar);
+                    } else {
+                        tma_4d(dst, &map_in, 0, t.x0 - 1, t.y - 1 + i, t.b, bar);
+                    }
                 }
                 s_a = s_e + 1;
             }
@@ -352,7 +370,7 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
             auto ready = [&](int q, int k, bool fresh) {
                 bool got = true;
                 if (fresh && k >= ACCS) got = mbar_wait(smem_u32(&acc_empty[acc_of(k)]), (uint32_t)((k / ACCS - 1) & 1));
-                got = mbar_wait(smem_u32(&row_full[q % RING]), (uint32_t)((q / RING) & 1)) && got;
+                got = mbar_wait(smem_u32(&row_full[q % ring]), (uint32_t)((q / ring) & 1)) && got;
                 __syncwarp();
                 fence_after();
                 if (!got) ok = false;
@@ -362,10 +380,10 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
             for (int s_a = s0; s_a < s1;) {
                 const int s_e = run_end(s_a, s1, H), R = s_e - s_a + 1;
                 for (int i = 0; i < R + 2; ++i, ++q) {
-                    const int slot = q % RING;
+                    const int slot = q % ring;
                     const int lo = i > 2 ? i - 2 : 0, hi = i < R ? i : R - 1;   // output rows this row adds to
                     const bool fresh = i < R;                                     // row i starts here (dy = 0)
-                    const uint64_t a0 = sdesc_sw128(sA + (uint32_t)(slot * A_ROW));
+                    const uint64_t a0 = sdesc_sw128(sA + (uint32_t)slot * slot_bytes);
                     // output rows hi, hi - 1, .. lo (accumulators ascending, dy = i - hi ascending) as
                     // one or, where the accumulator ring wraps, two MMAs
                     const int first = acc_of(k0 + hi), cnt = hi - lo + 1;
@@ -378,18 +396,18 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
                     mma_bf16(d1, a0, w1, fresh ? idesc_n(1) : i1, fresh ? 0u : 1u);
                     if (fresh && n1 > 1) mma_bf16(d1 + 64, a0, w1 + (uint64_t)(B_TAP >> 4), idesc_n(n1 - 1), 1u);
                     if (n2) mma_bf16(tmem, a0, w2, i2, 1u);
-                    // pixel m of the strip reads halo pixel m + dx (dx = t / 4 rows later);
+                    // pixel m of the strip reads halo pixel m + dx (dx = t / 4 rows later; FOLD: its copy);
                     // 16 channels (32 bytes of each row) per MMA
                     auto taps = [&](int t0, int t1) {
                         if (n2 == 0) {
 #pragma unroll
                             for (int t = t0; t < t1; ++t)
-                                mma_bf16(d1, a0 + (uint64_t)(((t / 4) * 128 + (t % 4) * 32) >> 4),
+                                mma_bf16(d1, a0 + (uint64_t)(((t / 4) * dx_bytes + (t % 4) * 32) >> 4),
                                          w1 + (uint64_t)(((t / 4) * 3 * B_TAP + (t % 4) * 32) >> 4), i1, 1u);
                         } else {
 #pragma unroll
                             for (int t = t0; t < t1; ++t) {
-                                const uint64_t ad = a0 + (uint64_t)(((t / 4) * 128 + (t % 4) * 32) >> 4);
+                                const uint64_t ad = a0 + (uint64_t)(((t / 4) * dx_bytes + (t % 4) * 32) >> 4);
                                 const uint64_t wo = (uint64_t)(((t / 4) * 3 * B_TAP + (t % 4) * 32) >> 4);
                                 mma_bf16(d1, ad, w1 + wo, i1, 1u);
                                 mma_bf16(tmem, ad, w2 + wo, i2, 1u);
@@ -419,7 +437,7 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
         auto load_mask = [&](int s) {
             const Strip t = strip_of(s, H, nx);
             mbar_expect_tx(smem_u32(&mask_full[g]), O_BYTES);
-            tma_4d(buf, &map_mask, 0, t.x0, t.y, t.b, smem_u32(&mask_full[g]));
+            tma_4d(buf, &map_mask, 0, t.x0, t.y, ib * t.b, smem_u32(&mask_full[g]));
         };
         if (leader) pdl_wait();   // the mask, and the buffer the output replaces, belong to earlier kernels
         if (MODE == 1 && leader && s0 + g < s1) load_mask(s0 + g);
@@ -465,7 +483,7 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
             named_bar(1 + g, 128);
             if (leader) {
                 const Strip t = strip_of(s0 + k, H, nx);
-                tma_store_4d(&map_out, buf, 0, t.x0, t.y, t.b);
+                tma_store_4d(&map_out, buf, 0, t.x0, t.y, ib * t.b);
                 if (MODE == 1 && s0 + k + EPI_GROUPS < s1) {
                     tma_store_read_wait();
                     load_mask(s0 + k + EPI_GROUPS);
@@ -739,8 +757,10 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
 namespace dgct {
 
 int conv64_tc_init() {
-    DGCT_CUDA(cudaFuncSetAttribute(tc::k_conv64_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM));
-    DGCT_CUDA(cudaFuncSetAttribute(tc::k_conv64_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM));
+    const void* convs[] = {(const void*)tc::k_conv64_tc<0, false>, (const void*)tc::k_conv64_tc<1, false>,
+                           (const void*)tc::k_conv64_tc<0, true>, (const void*)tc::k_conv64_tc<1, true>};
+    for (const void* k : convs)
+        DGCT_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM));
     DGCT_CUDA(cudaFuncSetAttribute(tc::k_wgrad64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::WG_SMEM));
     return DGAMP_CT_OK;
 }
@@ -779,7 +799,11 @@ static int encode(CUtensorMap* map, cuuint32_t rank, const void* base, const cuu
 int launch_conv64_tc(int mode, const void* in, const void* wk_all, int layers, int layer, const float* bias,
                      const void* mask, void* out, int B, int H, int W, int grid_cap, unsigned* err, cudaStream_t st,
                      unsigned long long stall_ns) {
-    const long long nstrips = (long long)B * H * ((W + tc::M - 1) / tc::M);
+    // rows of at most half a strip are taken two images at a time: 64-pixel rows as they are cost a whole
+    // strip each (32 patches of 64 x 64, the training pass 891 -> 847 us; bound by the L2 reads
+    // of the three copies)
+    const bool fold = W <= tc::M / 2 && B > 1;
+    const long long nstrips = (long long)(fold ? (B + 1) / 2 : B) * H * ((W + tc::M - 1) / tc::M);
     if (nstrips <= 0) return DGAMP_CT_OK;
     if (layer < 0 || layer >= layers) return DGAMP_CT_ERR_INVALID_ARG;
     CUtensorMap map_in, map_w, map_out, map_mask;
@@ -787,8 +811,9 @@ int launch_conv64_tc(int mode, const void* in, const void* wk_all, int layers, i
         const cuuint64_t dims[4] = {64, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {128, (cuuint64_t)W * 128, (cuuint64_t)H * W * 128};
         const cuuint32_t box[4] = {64, (cuuint32_t)tc::HWL, 1, 1};
-        DGCT_TRY(encode(&map_in, 4, in, dims, strides, box));
-        const cuuint32_t strip[4] = {64, (cuuint32_t)tc::M, 1, 1};
+        const cuuint32_t whole[4] = {64, (cuuint32_t)tc::M, 1, 1}, pair[4] = {64, (cuuint32_t)tc::M / 2, 1, 2};
+        const cuuint32_t* strip = fold ? pair : whole;
+        DGCT_TRY(encode(&map_in, 4, in, dims, strides, fold ? pair : box));
         DGCT_TRY(encode(&map_out, 4, out, dims, strides, strip));
         DGCT_TRY(encode(&map_mask, 4, mode == 1 ? mask : in, dims, strides, strip));
     }
@@ -803,7 +828,9 @@ int launch_conv64_tc(int mode, const void* in, const void* wk_all, int layers, i
     const int cap = grid_cap > 0 ? grid_cap : 1;
     const int per = (int)((nstrips + cap - 1) / cap);
     const int grid = (int)((nstrips + per - 1) / per);
-    DGCT_CUDA(launch_pdl(mode == 0 ? tc::k_conv64_tc<0> : tc::k_conv64_tc<1>, dim3(grid), dim3(tc::THREADS), tc::SMEM, st,
+    const auto kernel = fold ? (mode == 0 ? tc::k_conv64_tc<0, true> : tc::k_conv64_tc<1, true>)
+                             : (mode == 0 ? tc::k_conv64_tc<0, false> : tc::k_conv64_tc<1, false>);
+    DGCT_CUDA(launch_pdl(kernel, dim3(grid), dim3(tc::THREADS), tc::SMEM, st,
                          map_in, map_w, map_out, map_mask, layer, bias, B, H, W, per, err, stall_ns));
     return DGAMP_CT_OK;
 }
