@@ -82,17 +82,9 @@ k_fan_project(const T* __restrict__ XR, const T* __restrict__ XC, int ldp, int n
         const int len = (n + kFanSeg - 1) / kFanSeg;
         s0 = max(s0, seg * len);
         s1 = min(s1, seg * len + len - 1);
-        if (s0 <= s1) {
-            long long pos = R.P0 + (long long)s0 * R.PSTEP;
-            const T* __restrict__ line = B + (size_t)s0 * ldp + kPad;
-            for (int s = s0; s <= s1; ++s, pos += R.PSTEP, line += ldp) {
-                int i0;
-                float f;
-                joseph_tap(pos, i0, f);
-                const float x0 = ldf(line + i0), x1 = ldf(line + i0 + 1);
-                acc += fmaf(f, x1 - x0, x0);
-            }
-        }
+        if (s0 <= s1)
+            acc = joseph_march<8>(B, R.P0 + (long long)s0 * R.PSTEP + ((long long)(s0 * ldp + kPad) << 32), R.PSTEP, ldp,
+                               s1 - s0 + 1);
     }
     red[seg][lane] = acc;
     __syncthreads();

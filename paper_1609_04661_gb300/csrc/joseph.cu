@@ -87,18 +87,9 @@ __device__ __forceinline__ void project_block(const T* __restrict__ XR, const T*
         const int len = (n + kPjSeg - 1) / kPjSeg;
         s0 = max(s0, seg * len);
         s1 = min(s1, seg * len + len - 1);
-        if (s0 <= s1) {
-            long long pos = joseph_pos(c, d, s0);
-            const T* __restrict__ line = B + (size_t)s0 * ldp + kPad;
-#pragma unroll 4
-            for (int s = s0; s <= s1; ++s, pos += c.PSTEP, line += ldp) {
-                int i0;
-                float f;
-                joseph_tap(pos, i0, f);
-                const float x0 = ldf(line + i0), x1 = ldf(line + i0 + 1);
-                acc += fmaf(f, x1 - x0, x0);
-            }
-        }
+        if (s0 <= s1)
+            acc = joseph_march<8>(B, joseph_pos(c, d, s0) + ((long long)(s0 * ldp + kPad) << 32), c.PSTEP, ldp,
+                               s1 - s0 + 1);
     }
     red[seg][lane] = acc;
     __syncthreads();
