@@ -158,6 +158,26 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
+// Rows a warp still has to compute in step k (from 0) of a launch: the rows
+// kept at the end depend on rows k + 1 .. RH - k - 2 of this step's duals, so a
+// warp whose rows lie outside skips the step (its q also serves the row above
+// it); the results are the same.  With two rows per thread the special-function
+// unit and the issue slots of a 64-row region lose a sixth of their work
+// (30-iteration solve 2219 -> 2196 us).  With four or eight rows a block has
+// few warps and the branches cost more than the skipped work gives (batch of 12
+// slices 9820 -> 10090 us), so there every warp takes every step.
+struct TvActive {
+    bool q, p;
+};
+template <int WY, int V>
+__device__ __forceinline__ TvActive tv_active_rows(int w, int k) {
+    const int top = w * V, bottom = top + V - 1, RH = WY * V;
+    TvActive a;
+    a.p = V > 2 || (bottom > k && top < RH - 1 - k);
+    a.q = V > 2 || (bottom > k && top <= RH - 1 - k);
+    return a;
+}
+
 template <int WY, int KB, bool BORDER, int V = kTvV>
 __device__ __forceinline__ void tv_region_steps(float (&px)[V][kTvU], float (&py)[V][kTvU],
                                                 const float (&rl)[V][kTvU], unsigned inside, unsigned lastc,
@@ -171,61 +191,66 @@ __device__ __forceinline__ void tv_region_steps(float (&px)[V][kTvU], float (&py
 #pragma unroll 1
     for (int k = 0; k < KB; ++k) {
         // q = div p - r / lambda  (zero outside the image)
+        const TvActive on = tv_active_rows<WY, V>(w, k);
+        if (on.q) {
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
+            for (int v = 0; v < V; ++v) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                float pxl;
-                if (u > 0) {
-                    pxl = px[v][u - 1];
-                } else {
-                    const float t = __shfl_up_sync(0xffffffffu, px[v][U - 1], 1);
-                    pxl = lane > 0 ? t : 0.f;
+                for (int u = 0; u < U; ++u) {
+                    float pxl;
+                    if (u > 0) {
+                        pxl = px[v][u - 1];
+                    } else {
+                        const float t = __shfl_up_sync(0xffffffffu, px[v][U - 1], 1);
+                        pxl = lane > 0 ? t : 0.f;
+                    }
+                    const float pyu = v > 0 ? py[v - 1][u] : (w > 0 ? e_py[w - 1][u][lane] : 0.f);
+                    float qq = (px[v][u] - pxl + py[v][u] - pyu) - rl[v][u];
+                    if (BORDER && !((inside >> (v * U + u)) & 1u)) qq = 0.f;
+                    q[v][u] = qq;
                 }
-                const float pyu = v > 0 ? py[v - 1][u] : (w > 0 ? e_py[w - 1][u][lane] : 0.f);
-                float qq = (px[v][u] - pxl + py[v][u] - pyu) - rl[v][u];
-                if (BORDER && !((inside >> (v * U + u)) & 1u)) qq = 0.f;
-                q[v][u] = qq;
             }
-        }
 #pragma unroll
-        for (int u = 0; u < U; ++u) e_q[w][u][lane] = q[0][u];
+            for (int u = 0; u < U; ++u) e_q[w][u][lane] = q[0][u];
+        }
         __syncthreads();
-        // p <- (p + tau grad q) / (1 + tau |grad q|)  (grad q = 0 across the last row/column)
+        if (on.p) {
+            // p <- (p + tau grad q) / (1 + tau |grad q|)  (grad q = 0 across the last row/column)
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
+            for (int v = 0; v < V; ++v) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                float qr;
-                if (u + 1 < U) {
-                    qr = q[v][u + 1];
-                } else {
-                    const float t = __shfl_down_sync(0xffffffffu, q[v][0], 1);
-                    qr = lane < 31 ? t : 0.f;
-                }
-                const float qd = v + 1 < V ? q[v + 1][u] : (w + 1 < WY ? e_q[w + 1][u][lane] : 0.f);
-                float gx = qr - q[v][u];
-                float gy = qd - q[v][u];
-                bool upd = true;
-                if (BORDER) {
-                    const int bit = v * U + u;
-                    upd = (inside >> bit) & 1u;
-                    if ((lastc >> bit) & 1u) gx = 0.f;
-                    if ((lastr >> bit) & 1u) gy = 0.f;
-                }
-                if (upd) {
-                    // |grad q| and 1 / (1 + tau |grad q|) by the hardware's approximate
-                    // square root and reciprocal (sqrt(0) = 0; the denominator is >= 1)
-                    const float g2 = fmaf(gx, gx, gy * gy);
-                    const float nrm = sqrt_approx(g2);
-                    const float inv = rcp_approx(fmaf(kTau, nrm, 1.f));
-                    px[v][u] = fmaf(kTau, gx, px[v][u]) * inv;
-                    py[v][u] = fmaf(kTau, gy, py[v][u]) * inv;
+                for (int u = 0; u < U; ++u) {
+                    float qr;
+                    if (u + 1 < U) {
+                        qr = q[v][u + 1];
+                    } else {
+                        const float t = __shfl_down_sync(0xffffffffu, q[v][0], 1);
+                        qr = lane < 31 ? t : 0.f;
+                    }
+                    const float qd = v + 1 < V ? q[v + 1][u] : (w + 1 < WY ? e_q[w + 1][u][lane] : 0.f);
+                    float gx = qr - q[v][u];
+                    float gy = qd - q[v][u];
+                    bool upd = true;
+                    if (BORDER) {
+                        const int bit = v * U + u;
+                        upd = (inside >> bit) & 1u;
+                        if ((lastc >> bit) & 1u) gx = 0.f;
+                        if ((lastr >> bit) & 1u) gy = 0.f;
+                    }
+                    if (upd) {
+                        // |grad q| and 1 / (1 + tau |grad q|) by the hardware's approximate
+                        // square root and reciprocal (sqrt(0) = 0; the denominator is >= 1)
+                        const float g2 = fmaf(gx, gx, gy * gy);
+                        const float nrm = sqrt_approx(g2);
+                        const float inv = rcp_approx(fmaf(kTau, nrm, 1.f));
+                        px[v][u] = fmaf(kTau, gx, px[v][u]) * inv;
+                        py[v][u] = fmaf(kTau, gy, py[v][u]) * inv;
+                    }
                 }
             }
-        }
 #pragma unroll
-        for (int u = 0; u < U; ++u) e_py[w][u][lane] = py[V - 1][u];
+            for (int u = 0; u < U; ++u) e_py[w][u][lane] = py[V - 1][u];
+        }
         __syncthreads();
     }
 }
@@ -459,60 +484,65 @@ __device__ __forceinline__ void tv_region_steps2(float2 (&px)[V][kTvU], float2 (
 #pragma unroll 1
     for (int k = 0; k < KB; ++k) {
         // q = div p - r / lambda  (zero outside the image)
+        const TvActive on = tv_active_rows<WY, V>(w, k);
+        if (on.q) {
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
+            for (int v = 0; v < V; ++v) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                float2 pxl;
-                if (u > 0) {
-                    pxl = px[v][u - 1];
-                } else {
-                    const float2 t = shfl_up2(px[v][U - 1], 1);
-                    pxl = lane > 0 ? t : zero;
+                for (int u = 0; u < U; ++u) {
+                    float2 pxl;
+                    if (u > 0) {
+                        pxl = px[v][u - 1];
+                    } else {
+                        const float2 t = shfl_up2(px[v][U - 1], 1);
+                        pxl = lane > 0 ? t : zero;
+                    }
+                    const float2 pyu = v > 0 ? py[v - 1][u] : (w > 0 ? e_py[w - 1][u][lane] : zero);
+                    float2 qq = sub2(sub2(add2(sub2(px[v][u], pxl), py[v][u]), pyu), rl[v][u]);
+                    if (BORDER && !((inside >> (v * U + u)) & 1u)) qq = zero;
+                    q[v][u] = qq;
                 }
-                const float2 pyu = v > 0 ? py[v - 1][u] : (w > 0 ? e_py[w - 1][u][lane] : zero);
-                float2 qq = sub2(sub2(add2(sub2(px[v][u], pxl), py[v][u]), pyu), rl[v][u]);
-                if (BORDER && !((inside >> (v * U + u)) & 1u)) qq = zero;
-                q[v][u] = qq;
             }
-        }
 #pragma unroll
-        for (int u = 0; u < U; ++u) e_q[w][u][lane] = q[0][u];
+            for (int u = 0; u < U; ++u) e_q[w][u][lane] = q[0][u];
+        }
         __syncthreads();
-        // p <- (p + tau grad q) / (1 + tau |grad q|)  (grad q = 0 across the last row/column)
+        if (on.p) {
+            // p <- (p + tau grad q) / (1 + tau |grad q|)  (grad q = 0 across the last row/column)
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
+            for (int v = 0; v < V; ++v) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                float2 qr;
-                if (u + 1 < U) {
-                    qr = q[v][u + 1];
-                } else {
-                    const float2 t = shfl_down2(q[v][0], 1);
-                    qr = lane < 31 ? t : zero;
-                }
-                const float2 qd = v + 1 < V ? q[v + 1][u] : (w + 1 < WY ? e_q[w + 1][u][lane] : zero);
-                float2 gx = sub2(qr, q[v][u]);
-                float2 gy = sub2(qd, q[v][u]);
-                bool upd = true;
-                if (BORDER) {
-                    const int bit = v * U + u;
-                    upd = (inside >> bit) & 1u;
-                    if ((lastc >> bit) & 1u) gx = zero;
-                    if ((lastr >> bit) & 1u) gy = zero;
-                }
-                if (upd) {
-                    const float2 g2 = fma2(gx, gx, mul2(gy, gy));
-                    const float2 nrm = make_float2(sqrt_approx(g2.x), sqrt_approx(g2.y));
-                    const float2 den = fma2(tau, nrm, one);
-                    const float2 inv = make_float2(rcp_approx(den.x), rcp_approx(den.y));
-                    px[v][u] = mul2(fma2(tau, gx, px[v][u]), inv);
-                    py[v][u] = mul2(fma2(tau, gy, py[v][u]), inv);
+                for (int u = 0; u < U; ++u) {
+                    float2 qr;
+                    if (u + 1 < U) {
+                        qr = q[v][u + 1];
+                    } else {
+                        const float2 t = shfl_down2(q[v][0], 1);
+                        qr = lane < 31 ? t : zero;
+                    }
+                    const float2 qd = v + 1 < V ? q[v + 1][u] : (w + 1 < WY ? e_q[w + 1][u][lane] : zero);
+                    float2 gx = sub2(qr, q[v][u]);
+                    float2 gy = sub2(qd, q[v][u]);
+                    bool upd = true;
+                    if (BORDER) {
+                        const int bit = v * U + u;
+                        upd = (inside >> bit) & 1u;
+                        if ((lastc >> bit) & 1u) gx = zero;
+                        if ((lastr >> bit) & 1u) gy = zero;
+                    }
+                    if (upd) {
+                        const float2 g2 = fma2(gx, gx, mul2(gy, gy));
+                        const float2 nrm = make_float2(sqrt_approx(g2.x), sqrt_approx(g2.y));
+                        const float2 den = fma2(tau, nrm, one);
+                        const float2 inv = make_float2(rcp_approx(den.x), rcp_approx(den.y));
+                        px[v][u] = mul2(fma2(tau, gx, px[v][u]), inv);
+                        py[v][u] = mul2(fma2(tau, gy, py[v][u]), inv);
+                    }
                 }
             }
-        }
 #pragma unroll
-        for (int u = 0; u < U; ++u) e_py[w][u][lane] = py[V - 1][u];
+            for (int u = 0; u < U; ++u) e_py[w][u][lane] = py[V - 1][u];
+        }
         __syncthreads();
     }
 }
