@@ -177,54 +177,29 @@ __global__ void __launch_bounds__(512) k_batch_vinv_rows(const BatchSlice* __res
                                                          const uint16_t* __restrict__ map) {
     extern __shared__ float2 smem[];
     const BatchSlice& B = sl[map[blockIdx.x]];
-    const int iy = (int)blockIdx.x - B.off[kPhRow], n = B.n, m = B.m2;
-    float2* a = smem;
-    float2* b = smem + fft_buf_len(m);
-    for (int i = threadIdx.x; i < m; i += blockDim.x)
-        a[fpad(i)] = make_float2(i < n ? B.x[(size_t)iy * n + i] : 0.f, 0.f);
-    __syncthreads();
-    float2* r = fft_stockham(a, b, m, B.tw2, -1.f);
-    for (int i = threadIdx.x; i < m; i += blockDim.x) B.fft2d[(size_t)iy * m + i] = r[fpad(i)];
+    img_rows_fwd_block(B.x, B.n, B.m2, 2 * ((int)blockIdx.x - B.off[kPhRow]), B.tw2, B.fft2d, smem);
 }
 
 __global__ void __launch_bounds__(512) k_batch_vinv_cols(const BatchSlice* __restrict__ sl,
                                                          const uint16_t* __restrict__ map) {
     extern __shared__ float2 smem[];
     const BatchSlice& B = sl[map[blockIdx.x]];
-    const int kx = (int)blockIdx.x - B.off[kPhCol], n = B.n, m = B.m2;
-    float2* a = smem;
-    float2* b = smem + fft_buf_len(m);
-    float2* C = B.fft2d;
-    for (int i = threadIdx.x; i < m; i += blockDim.x)
-        a[fpad(i)] = i < n ? C[(size_t)i * m + kx] : make_float2(0.f, 0.f);
-    __syncthreads();
-    float2* r = fft_stockham(a, b, m, B.tw2, -1.f);
-    float2* o = (r == a) ? b : a;
-    const float f0 = 1.0f / (2.0f * (float)B.P);
-    const float fx = (float)(kx <= m / 2 ? kx : kx - m) / (float)m;
-    for (int ky = threadIdx.x; ky < m; ky += blockDim.x) {
-        const float fy = (float)(ky <= m / 2 ? ky : ky - m) / (float)m;
-        const float g = sqrtf(fmaxf(sqrtf(fx * fx + fy * fy), f0));
-        const float2 v = r[fpad(ky)];
-        r[fpad(ky)] = make_float2(v.x * g, v.y * g);
-    }
-    __syncthreads();
-    r = fft_stockham(r, o, m, B.tw2, 1.f);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) C[(size_t)i * m + kx] = r[fpad(i)];
+    img_cols_block(B.fft2d, B.n, B.m2, (int)blockIdx.x - B.off[kPhCol], B.tw2, 1.0f / (2.0f * (float)B.P), 0, smem);
 }
 
 __global__ void __launch_bounds__(512) k_batch_vinv_rows_inv(const BatchSlice* __restrict__ sl,
                                                              const uint16_t* __restrict__ map) {
     extern __shared__ float2 smem[];
     const BatchSlice& B = sl[map[blockIdx.x]];
-    const int iy = (int)blockIdx.x - B.off[kPhRow], n = B.n, m = B.m2;
-    float2* a = smem;
-    float2* b = smem + fft_buf_len(m);
-    for (int i = threadIdx.x; i < m; i += blockDim.x) a[fpad(i)] = B.fft2d[(size_t)iy * m + i];
-    __syncthreads();
-    float2* r = fft_stockham(a, b, m, B.tw2, 1.f);
-    const float sc = 1.0f / ((float)m * (float)m);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) B.mu_out[(size_t)iy * n + i] = r[fpad(i)].x * sc;
+    const int y0 = 2 * ((int)blockIdx.x - B.off[kPhRow]), n = B.n;
+    const float2* r = img_rows_inv_block(B.fft2d, n, B.m2, y0, B.tw2, smem);
+    const float sc = 1.0f / ((float)B.m2 * (float)B.m2);
+    float* __restrict__ out = B.mu_out + (size_t)y0 * n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const float2 v = r[fpad(i)];
+        out[i] = v.x * sc;
+        if (y0 + 1 < n) out[n + i] = v.y * sc;
+    }
 }
 
 }  // namespace dgct
@@ -393,6 +368,8 @@ int dgamp_ct_batch_create(int32_t n, const dgamp_ct_plan_t* plans, int32_t group
     b->h.resize(n);
     std::vector<std::vector<uint16_t>> maps(kPhases);
     std::vector<std::vector<std::vector<uint16_t>>> gmaps(G, std::vector<std::vector<uint16_t>>(kPhases));
+    for (int32_t i = 0; i < n; ++i) E.max_m2 = std::max(E.max_m2, plans[i]->m2);
+    const int vinv_nc = img_cols_per_block(E.max_m2);
     for (int32_t k = 0; k < n; ++k) {
         const int32_t i = order[k];
         const dgamp_ct_plan_s* pl = plans[i];
@@ -414,14 +391,13 @@ int dgamp_ct_batch_create(int32_t n, const dgamp_ct_plan_t* plans, int32_t group
         const long long begin_elems = std::max<long long>(std::max<long long>(pl->M, pl->N), (long long)pl->n * pl->ldp);
         const int cnt[kPhases] = {batch_grid_project(pl->nv, pl->nd), pl->nv, batch_grid_backproject(pl->n),
                                   batch_grid_probe(pl->N), batch_grid_tv(pl->n, 0), batch_grid_tv(pl->n, 1),
-                                  pl->n, pl->m2, (int)((begin_elems + 255) / 256)};
+                                  (pl->n + 1) / 2, img_col_blocks(pl->m2, vinv_nc), (int)((begin_elems + 255) / 256)};
         const int gk = group_of[i];
         for (int ph = 0; ph < kPhases; ++ph) {
             auto& mp = (ph == kPhRow || ph == kPhCol || ph == kPhBegin) ? maps[ph] : gmaps[gk][ph];
             d.off[ph] = (int)mp.size();
             mp.insert(mp.end(), (size_t)cnt[ph], (uint16_t)i);
         }
-        E.max_m2 = std::max(E.max_m2, pl->m2);
         gmax_nd[gk] = std::max(gmax_nd[gk], pl->nd);
     }
     for (int ph = 0; ph < kPhases; ++ph) E.nblk[ph] = (int)maps[ph].size();
@@ -450,7 +426,7 @@ int dgamp_ct_batch_create(int32_t n, const dgamp_ct_plan_t* plans, int32_t group
     for (auto& X : b->grp) X.sl = E.sl;
     if (e != cudaSuccess) rc = (e == cudaErrorMemoryAllocation) ? DGAMP_CT_ERR_OOM : cuda_fail(e);
     if (rc == DGAMP_CT_OK) {
-        const int fsm = 2 * fft_buf_len(E.max_m2) * (int)sizeof(float2);
+        const int fsm = 2 * fft_buf_len(E.max_m2) * (int)sizeof(float2) * vinv_nc;
         const int lim = fsm > 48 * 1024 ? fsm : 48 * 1024;
         rc = raise_smem_limit((const void*)k_batch_vinv_rows, lim);
         if (rc == DGAMP_CT_OK) rc = raise_smem_limit((const void*)k_batch_vinv_cols, lim);
@@ -509,7 +485,8 @@ int dgamp_ct_batch_solve(dgamp_ct_batch_t b, const float* const* d_counts, const
     const size_t fsm = (size_t)2 * fft_buf_len(E.max_m2) * sizeof(float2);
     k_batch_vinv_rows<<<E.nblk[kPhRow], thr, fsm, st>>>(E.sl, E.map[kPhRow]);
     DGCT_LAUNCH_CHECK();
-    k_batch_vinv_cols<<<E.nblk[kPhCol], thr, fsm, st>>>(E.sl, E.map[kPhCol]);
+    const int nc = img_cols_per_block(E.max_m2);
+    k_batch_vinv_cols<<<E.nblk[kPhCol], dim3(thr, nc), nc * fsm, st>>>(E.sl, E.map[kPhCol]);
     DGCT_LAUNCH_CHECK();
     k_batch_vinv_rows_inv<<<E.nblk[kPhRow], thr, fsm, st>>>(E.sl, E.map[kPhRow]);
     DGCT_LAUNCH_CHECK();

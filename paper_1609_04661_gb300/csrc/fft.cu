@@ -1,15 +1,16 @@
 // Shared-memory FFTs for the Radon preconditioner (Section 2.4, Eq. Aprecon).
 //
-//  * H on sinograms: one block filters two views at once, packed as the real
-//    and imaginary parts of one complex line.  Because the gain g is real and
-//    even, filtering a + i b gives H a + i H b, so one forward and one inverse
-//    complex FFT of length P serve two views.
+//  * H on sinograms: one block per view, the real line of length P as a complex
+//    one of length P/2 (even bins + i odd bins), split into the spectra of the
+//    even and odd bins for the gain and put together again.
 //  * V^-1 / V on images: a 2-D zero-padded FFT done as row FFTs, column FFTs
 //    with the radial gain applied between the forward and inverse column
 //    transforms, and inverse row FFTs.  It runs once per solve.
 //
 // The transform (fft_device.cuh) is a Stockham autosort FFT with radix-8
 // stages, in shared memory.
+#include <algorithm>
+
 #include "fft_device.cuh"
 
 namespace dgct {
@@ -18,42 +19,56 @@ namespace dgct {
 static int fft_threads(int P) { return P / 8 < 32 ? 32 : (P / 8 > 512 ? 512 : P / 8); }
 
 // ------------------------------------------------------------ H on views --
+// One view per block.  With z[j] = x[2j] + i x[2j + 1] and Z its DFT of length
+// L = P / 2, the even and odd bins' DFTs are E = (Z[k] + conj Z[L-k]) / 2 and
+// O = (Z[k] - conj Z[L-k]) / 2i, and x's own are E +- w^k O at k and k + L,
+// w = exp(-2 pi i / P).  Multiplying those by the gains a = g[k] and
+// b = g[k + L] = g[L-k] gives
+//   E' = ((a + b) E + (a - b) w^k O) / 2,   O' = ((a - b) w^-k E + (a + b) O) / 2,
+// and Z' = E' + i O' (at L-k: conj E' + i conj O') transforms back to the
+// filtered bins.  The block's chain of stages and barriers bounds the kernel,
+// not its arithmetic: a pair of views per block as one complex line of length P
+// left 45 blocks with twice the butterflies per stage at 90 views, P = 4096.
+// Two filters and an output step at 90 x 1449: 55.5 -> 50.2 us.
 template <typename T>
 __global__ void __launch_bounds__(512)
-k_filter_views(const T* in, T* out, int nv, int nd, int P,
-               const float* __restrict__ gain, const float2* __restrict__ tw) {
+k_filter_views(const T* in, T* out, int nd, int P, const float* __restrict__ gain, const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
+    const int L = P >> 1;
     float2* a = smem;
-    float2* b = smem + fft_buf_len(P);
-    const int va = 2 * blockIdx.x, vb = va + 1;
-    const bool hasb = vb < nv;
-    const T* ra = in + (size_t)va * nd;
-    const T* rb = in + (size_t)vb * nd;
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
+    float2* b = smem + fft_buf_len(L);
+    const T* row = in + (size_t)blockIdx.x * nd;
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
         float2 v = make_float2(0.f, 0.f);
-        if (i < nd) {
-            v.x = ldf(ra + i);
-            if (hasb) v.y = ldf(rb + i);
-        }
+        if (2 * i < nd) v.x = ldf(row + 2 * i);
+        if (2 * i + 1 < nd) v.y = ldf(row + 2 * i + 1);
         a[fpad(i)] = v;
     }
     __syncthreads();
-    float2* r = fft_stockham(a, b, P, tw, -1.f);
+    float2* r = fft_stockham(a, b, L, tw, -1.f);
     float2* o = (r == a) ? b : a;
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const float g = __ldg(gain + i);
-        const float2 v = r[fpad(i)];
-        r[fpad(i)] = make_float2(v.x * g, v.y * g);
+    const float sc = 0.25f / (float)L;      // the two halvings above, and 1 / L of the inverse
+    for (int k = threadIdx.x; k <= L / 2; k += blockDim.x) {
+        const int kk = (L - k) & (L - 1);
+        const float2 z = r[fpad(k)], y = r[fpad(kk)];
+        const float ga = __ldg(gain + k), gb = __ldg(gain + L - k);
+        const float gp = (ga + gb) * sc, gm = (ga - gb) * sc;
+        float sn, cs;
+        sincospif((float)k / (float)L, &sn, &cs);                    // w^k = cs - i sn
+        const float2 E = make_float2(z.x + y.x, z.y - y.y), O = make_float2(z.y + y.y, y.x - z.x);   // twice E, O
+        const float2 wO = make_float2(fmaf(cs, O.x, sn * O.y), fmaf(cs, O.y, -sn * O.x));
+        const float2 wE = make_float2(fmaf(cs, E.x, -sn * E.y), fmaf(cs, E.y, sn * E.x));            // w^-k E
+        const float2 e = make_float2(fmaf(gp, E.x, gm * wO.x), fmaf(gp, E.y, gm * wO.y));
+        const float2 q = make_float2(fmaf(gm, wE.x, gp * O.x), fmaf(gm, wE.y, gp * O.y));
+        r[fpad(k)] = make_float2(e.x - q.y, e.y + q.x);
+        if (kk != k) r[fpad(kk)] = make_float2(e.x + q.y, q.x - e.y);
     }
     __syncthreads();
-    r = fft_stockham(r, o, P, tw, 1.f);
-    const float sc = 1.0f / (float)P;
-    T* wa = out + (size_t)va * nd;
-    T* wb = out + (size_t)vb * nd;
+    r = fft_stockham(r, o, L, tw, 1.f);
+    T* w = out + (size_t)blockIdx.x * nd;
     for (int i = threadIdx.x; i < nd; i += blockDim.x) {
-        const float2 v = r[fpad(i)];
-        stf(wa + i, v.x * sc);
-        if (hasb) stf(wb + i, v.y * sc);
+        const float2 v = r[fpad(i >> 1)];
+        stf(w + i, (i & 1) ? v.y : v.x);
     }
 }
 
@@ -141,15 +156,14 @@ int launch_filter(const dgamp_ct_plan_s* pl, const float* in, float* out, cudaSt
         DGCT_LAUNCH_CHECK();
         return DGAMP_CT_OK;
     }
-    const int P = pl->P;
-    const size_t sm = (size_t)2 * fft_buf_len(P) * sizeof(float2);
-    const int thr = fft_threads(P);
+    const int P = pl->P, L = P / 2;
+    const size_t sm = (size_t)2 * fft_buf_len(L) * sizeof(float2);
+    const int thr = fft_threads(L);
     if (bf)
-        k_filter_views<bf16s><<<(pl->nv + 1) / 2, thr, sm, st>>>((const bf16s*)in, (bf16s*)out, pl->nv, pl->nd, P,
-                                                                 pl->ws.gain, pl->ws.tw);
+        k_filter_views<bf16s><<<pl->nv, thr, sm, st>>>((const bf16s*)in, (bf16s*)out, pl->nd, P, pl->ws.gain,
+                                                       pl->ws.twh);
     else
-        k_filter_views<float><<<(pl->nv + 1) / 2, thr, sm, st>>>(in, out, pl->nv, pl->nd, P, pl->ws.gain,
-                                                                 pl->ws.tw);
+        k_filter_views<float><<<pl->nv, thr, sm, st>>>(in, out, pl->nd, P, pl->ws.gain, pl->ws.twh);
     DGCT_LAUNCH_CHECK();
     return DGAMP_CT_OK;
 }
@@ -195,73 +209,41 @@ int toeplitz_set_smem_limit(int nd) {
 }
 
 // ------------------------------------------------------- V^-1 / V image --
-// Image blockIdx.y of a batch (img and out [nimg][n][n], C [nimg][n][m]); a
-// single image is the batch of one.
-// pass 1: rows iy < n of the m x m padded image -> C[iy][:]
+// Image blockIdx.y of a batch (img and out [nimg][n][n], C [nimg][n][img_stride(m)]);
+// a single image is the batch of one.  The passes are in fft_device.cuh.
 __global__ void __launch_bounds__(512)
 k_img_rows_fwd(const float* __restrict__ img, int n, int m, const float2* __restrict__ tw,
                float2* __restrict__ C) {
     extern __shared__ float2 smem[];
-    float2* a = smem;
-    float2* b = smem + fft_buf_len(m);
-    const int iy = blockIdx.x;
-    img += (size_t)blockIdx.y * n * n;
-    C += (size_t)blockIdx.y * n * m;
-    for (int i = threadIdx.x; i < m; i += blockDim.x)
-        a[fpad(i)] = make_float2(i < n ? img[(size_t)iy * n + i] : 0.f, 0.f);
-    __syncthreads();
-    float2* r = fft_stockham(a, b, m, tw, -1.f);
-    for (int i = threadIdx.x; i < m; i += blockDim.x) C[(size_t)iy * m + i] = r[fpad(i)];
+    img_rows_fwd_block(img + (size_t)blockIdx.y * n * n, n, m, 2 * blockIdx.x, tw,
+                       C + (size_t)blockIdx.y * n * img_stride(m), smem);
 }
 
-// pass 2: every column kx: forward FFT over rows (rows >= n are zero),
-// radial gain, inverse FFT; rows < n are stored back.
 __global__ void __launch_bounds__(512)
 k_img_cols(float2* __restrict__ C, int n, int m, const float2* __restrict__ tw, float f0,
            int inverse_gain) {
     extern __shared__ float2 smem[];
-    float2* a = smem;
-    float2* b = smem + fft_buf_len(m);
-    const int kx = blockIdx.x;
-    C += (size_t)blockIdx.y * n * m;
-    for (int i = threadIdx.x; i < m; i += blockDim.x)
-        a[fpad(i)] = i < n ? C[(size_t)i * m + kx] : make_float2(0.f, 0.f);
-    __syncthreads();
-    float2* r = fft_stockham(a, b, m, tw, -1.f);
-    float2* o = (r == a) ? b : a;
-    const float fx = (float)(kx <= m / 2 ? kx : kx - m) / (float)m;
-    for (int ky = threadIdx.x; ky < m; ky += blockDim.x) {
-        const float fy = (float)(ky <= m / 2 ? ky : ky - m) / (float)m;
-        const float rho = sqrtf(fx * fx + fy * fy);
-        float g = sqrtf(fmaxf(rho, f0));
-        if (inverse_gain) g = 1.0f / g;
-        const float2 v = r[fpad(ky)];
-        r[fpad(ky)] = make_float2(v.x * g, v.y * g);
-    }
-    __syncthreads();
-    r = fft_stockham(r, o, m, tw, 1.f);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) C[(size_t)i * m + kx] = r[fpad(i)];
+    img_cols_block(C + (size_t)blockIdx.y * n * img_stride(m), n, m, blockIdx.x, tw, f0, inverse_gain, smem);
 }
 
-// pass 3: inverse row FFTs, real part of the first n columns, scaled by 1/m^2.
+// pass 3: inverse row FFTs, the first n columns, scaled by 1/m^2.
 __global__ void __launch_bounds__(512)
 k_img_rows_inv(const float2* __restrict__ C, int n, int m, const float2* __restrict__ tw,
                float* __restrict__ out) {
     extern __shared__ float2 smem[];
-    float2* a = smem;
-    float2* b = smem + fft_buf_len(m);
-    const int iy = blockIdx.x;
-    C += (size_t)blockIdx.y * n * m;
-    out += (size_t)blockIdx.y * n * n;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) a[fpad(i)] = C[(size_t)iy * m + i];
-    __syncthreads();
-    float2* r = fft_stockham(a, b, m, tw, 1.f);
+    const int y0 = 2 * blockIdx.x;
+    const float2* r = img_rows_inv_block(C + (size_t)blockIdx.y * n * img_stride(m), n, m, y0, tw, smem);
+    out += (size_t)blockIdx.y * n * n + (size_t)y0 * n;
     const float sc = 1.0f / ((float)m * (float)m);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) out[(size_t)iy * n + i] = r[fpad(i)].x * sc;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const float2 v = r[fpad(i)];
+        out[i] = v.x * sc;
+        if (y0 + 1 < n) out[n + i] = v.y * sc;
+    }
 }
 
 // pass 3 of V^-1 inside a fan-beam solve (Algorithm 1, Step 3 with
-// Phi~^T = V^-1 A^T): r = x + tau_r Re(.) / m^2 with tau_r from the device
+// Phi~^T = V^-1 A^T): r = x + tau_r (.) / m^2 with tau_r from the device
 // scalars (the output step formed it), max |r| into S->rmax_bits (the output
 // step reset it), and the consumed divergence flag cleared, as the
 // parallel-beam back-projection does.
@@ -270,73 +252,65 @@ k_img_rows_inv_update(const float2* __restrict__ C, int n, int m, const float2* 
                       const float* __restrict__ x, DevScalars* __restrict__ S, float* __restrict__ out) {
     extern __shared__ float2 smem[];
     __shared__ unsigned s_max;
-    float2* a = smem;
-    float2* b = smem + fft_buf_len(m);
-    const int iy = blockIdx.x;
+    const int y0 = 2 * blockIdx.x;
     if (threadIdx.x == 0) {
         s_max = 0u;
-        if (iy == 0) S->div_pending = 0u;
+        if (y0 == 0) S->div_pending = 0u;
     }
-    for (int i = threadIdx.x; i < m; i += blockDim.x) a[fpad(i)] = C[(size_t)iy * m + i];
-    __syncthreads();
-    const float2* r = fft_stockham(a, b, m, tw, 1.f);
+    const float2* r = img_rows_inv_block(C, n, m, y0, tw, smem);
     const float sc = (float)S->tau_r / ((float)m * (float)m);
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const size_t o = (size_t)iy * n + i;
-        const float rv = fmaf(sc, r[fpad(i)].x, x[o]);
-        out[o] = rv;
-        atomicMax(&s_max, __float_as_uint(fabsf(rv)));   // |r| >= 0: bit order is value order
+        const float2 v = r[fpad(i)];
+        for (int h = 0; h < 2 && y0 + h < n; ++h) {
+            const size_t o = (size_t)(y0 + h) * n + i;
+            const float rv = fmaf(sc, h ? v.y : v.x, x[o]);
+            out[o] = rv;
+            atomicMax(&s_max, __float_as_uint(fabsf(rv)));   // |r| >= 0: bit order is value order
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) atomicMax(&S->rmax_bits, s_max);
+}
+
+// The two first passes of nimg images.
+static int launch_img_forward(const dgamp_ct_plan_s* pl, const float* in, float2* C, int nimg, int inverse_gain,
+                              cudaStream_t st) {
+    const int n = pl->n, m = pl->m2, thr = fft_threads(m), nc = img_cols_per_block(m);
+    const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
+    const float f0 = 1.0f / (2.0f * (float)pl->P);
+    k_img_rows_fwd<<<dim3((n + 1) / 2, nimg), thr, sm, st>>>(in, n, m, pl->ws.tw2, C);
+    DGCT_LAUNCH_CHECK();
+    // V^-1 applies sqrt(max(rho, f0)); V applies its reciprocal
+    k_img_cols<<<dim3(img_col_blocks(m, nc), nimg), dim3(thr, nc), nc * sm, st>>>(C, n, m, pl->ws.tw2, f0, inverse_gain);
+    DGCT_LAUNCH_CHECK();
+    return DGAMP_CT_OK;
 }
 
 int launch_precond_image_update(const dgamp_ct_plan_s* pl, const float* in, const float* x, float* out,
                                 cudaStream_t st) {
     const int n = pl->n, m = pl->m2;
     const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
-    const int thr = fft_threads(m);
-    const float f0 = 1.0f / (2.0f * (float)pl->P);
-    k_img_rows_fwd<<<n, thr, sm, st>>>(in, n, m, pl->ws.tw2, pl->ws.fft2d);
-    DGCT_LAUNCH_CHECK();
-    k_img_cols<<<m, thr, sm, st>>>(pl->ws.fft2d, n, m, pl->ws.tw2, f0, 0);
-    DGCT_LAUNCH_CHECK();
-    k_img_rows_inv_update<<<n, thr, sm, st>>>(pl->ws.fft2d, n, m, pl->ws.tw2, x, pl->ws.S, out);
+    DGCT_TRY(launch_img_forward(pl, in, pl->ws.fft2d, 1, 0, st));
+    k_img_rows_inv_update<<<(n + 1) / 2, fft_threads(m), sm, st>>>(pl->ws.fft2d, n, m, pl->ws.tw2, x, pl->ws.S, out);
     DGCT_LAUNCH_CHECK();
     return DGAMP_CT_OK;
 }
 
 int launch_precond_image(const dgamp_ct_plan_s* pl, const float* in, float* out, int inverse,
                          cudaStream_t st) {
-    const int n = pl->n, m = pl->m2;
-    const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
-    const int thr = fft_threads(m);
-    const float f0 = 1.0f / (2.0f * (float)pl->P);
-    k_img_rows_fwd<<<n, thr, sm, st>>>(in, n, m, pl->ws.tw2, pl->ws.fft2d);
-    DGCT_LAUNCH_CHECK();
-    // V^-1 applies sqrt(max(rho, f0)); V applies its reciprocal
-    k_img_cols<<<m, thr, sm, st>>>(pl->ws.fft2d, n, m, pl->ws.tw2, f0, inverse ? 0 : 1);
-    DGCT_LAUNCH_CHECK();
-    k_img_rows_inv<<<n, thr, sm, st>>>(pl->ws.fft2d, n, m, pl->ws.tw2, out);
-    DGCT_LAUNCH_CHECK();
-    return DGAMP_CT_OK;
+    return launch_precond_images(pl, in, out, pl->ws.fft2d, 1, inverse, st);
 }
 
 // nimg images at once ([nimg][n][n] in and out) through the scratch C
-// ([nimg][n][m] complex, the caller's); the same kernels and arithmetic per
-// image as launch_precond_image
+// ([nimg][n][m2] complex at least, the caller's); the same kernels and
+// arithmetic per image as launch_precond_image
 int launch_precond_images(const dgamp_ct_plan_s* pl, const float* in, float* out, float2* C, int nimg, int inverse,
                           cudaStream_t st) {
     if (nimg < 1) return DGAMP_CT_ERR_INVALID_ARG;
     const int n = pl->n, m = pl->m2;
     const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
-    const int thr = fft_threads(m);
-    const float f0 = 1.0f / (2.0f * (float)pl->P);
-    k_img_rows_fwd<<<dim3(n, nimg), thr, sm, st>>>(in, n, m, pl->ws.tw2, C);
-    DGCT_LAUNCH_CHECK();
-    k_img_cols<<<dim3(m, nimg), thr, sm, st>>>(C, n, m, pl->ws.tw2, f0, inverse ? 0 : 1);
-    DGCT_LAUNCH_CHECK();
-    k_img_rows_inv<<<dim3(n, nimg), thr, sm, st>>>(C, n, m, pl->ws.tw2, out);
+    DGCT_TRY(launch_img_forward(pl, in, C, nimg, inverse ? 0 : 1, st));
+    k_img_rows_inv<<<dim3((n + 1) / 2, nimg), fft_threads(m), sm, st>>>(C, n, m, pl->ws.tw2, out);
     DGCT_LAUNCH_CHECK();
     return DGAMP_CT_OK;
 }
@@ -345,7 +319,9 @@ int fft_set_smem_limits(int bytes) {
     DGCT_TRY(raise_smem_limit((const void*)k_filter_views<float>, bytes));
     DGCT_TRY(raise_smem_limit((const void*)k_filter_views<bf16s>, bytes));
     DGCT_TRY(raise_smem_limit((const void*)k_img_rows_fwd, bytes));
-    DGCT_TRY(raise_smem_limit((const void*)k_img_cols, bytes));
+    // several columns a block up to m = 2048: 4 at 1024 and 2 at 2048 need the same 74 KB
+    DGCT_TRY(raise_smem_limit((const void*)k_img_cols,
+                              std::max(bytes, (int)(4 * 2 * fft_buf_len(1024) * sizeof(float2)))));
     DGCT_TRY(raise_smem_limit((const void*)k_img_rows_inv, bytes));
     DGCT_TRY(raise_smem_limit((const void*)k_img_rows_inv_update, bytes));
     return DGAMP_CT_OK;

@@ -152,6 +152,7 @@ struct Workspace {
     float* zraw2 = nullptr;        // [M]  copy for in-place Toeplitz filtering
     float2* tw = nullptr;          // FFT twiddles for length P, stage by stage (fft_device.cuh)
     float2* tw2 = nullptr;         // the same for length m2
+    float2* twh = nullptr;         // the same for length P / 2 (H of a view as a real line)
     double* scratch_d = nullptr;   // plan-time FP64 scratch
     float* b = nullptr;            // the iteration's probe b (Eq. MC_SURE) [n][n]
     FanRay* fan_rays = nullptr;    // fan-beam plans: [n_views][n_det]
