@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kC1Threads)
 k_conv_first(const float* __restrict__ r, const float* __restrict__ sigma, int B, int H, int W,
              const float* __restrict__ w0, const float* __restrict__ b0,
              const bf16* __restrict__ mask, bf16* __restrict__ a1, float* __restrict__ u_out) {
-    __shared__ float sw[9 * CH + CH];
+    __shared__ __align__(16) float sw[9 * CH + CH];
     __shared__ __align__(16) bf16 stage[kC1Threads / 32][32 * PSTR];   // one warp's 32 rows
     for (int i = threadIdx.x; i < 9 * CH; i += blockDim.x) sw[i] = w0[i];
     for (int i = threadIdx.x; i < CH; i += blockDim.x) sw[9 * CH + i] = b0 ? b0[i] : 0.f;
@@ -91,15 +91,27 @@ k_conv_first(const float* __restrict__ r, const float* __restrict__ sigma, int B
         __align__(16) bf16 v[8];
         __align__(16) bf16 mk[8];
         if (mask) *reinterpret_cast<uint4*>(mk) = *reinterpret_cast<const uint4*>(row);
+        // channels in packed FP32 pairs (one instruction for both, each rounded as fmaf rounds it)
+        float2 acc[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] = *reinterpret_cast<const float2*>(sw + 9 * CH + c0 + 2 * j);
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const float4 wa = *reinterpret_cast<const float4*>(sw + t * CH + c0);
+            const float4 wb = *reinterpret_cast<const float4*>(sw + t * CH + c0 + 4);
+            const float2 u2 = make_float2(u[t], u[t]);
+            acc[0] = __ffma2_rn(u2, make_float2(wa.x, wa.y), acc[0]);
+            acc[1] = __ffma2_rn(u2, make_float2(wa.z, wa.w), acc[1]);
+            acc[2] = __ffma2_rn(u2, make_float2(wb.x, wb.y), acc[2]);
+            acc[3] = __ffma2_rn(u2, make_float2(wb.z, wb.w), acc[3]);
+        }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            float acc = sw[9 * CH + c0 + j];
-#pragma unroll
-            for (int t = 0; t < 9; ++t) acc = fmaf(u[t], sw[t * CH + c0 + j], acc);
+            const float a = (j & 1) ? acc[j >> 1].y : acc[j >> 1].x;
             if (mask)
-                v[j] = __float2bfloat16_rn(__bfloat162float(mk[j]) > 0.f ? acc : 0.f);
+                v[j] = __float2bfloat16_rn(__bfloat162float(mk[j]) > 0.f ? a : 0.f);
             else
-                v[j] = __float2bfloat16_rn(fmaxf(acc, 0.f));
+                v[j] = __float2bfloat16_rn(fmaxf(a, 0.f));
         }
         *reinterpret_cast<uint4*>(row) = *reinterpret_cast<const uint4*>(v);
     }
