@@ -23,7 +23,7 @@ int cuda_fail(cudaError_t e) {
 static void free_ws(Workspace& w) {
     void* ptrs[] = {w.XR, w.XC, w.x, w.r, w.b, w.p, w.zraw, w.z, w.s, w.hs, w.y, w.fft2d, w.partial,
                     w.partial_div, w.S, w.log, w.vc, w.gain, w.tw, w.tw2, w.twh, w.scratch_d, w.hx, w.zraw2,
-                    w.fan_rays, w.fan_views, w.pj_order, w.pj_part};
+                    w.fan_rays, w.fan_views, w.fan_gw, w.pj_order, w.pj_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     w = Workspace{};

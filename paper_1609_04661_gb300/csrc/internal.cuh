@@ -83,6 +83,7 @@ struct FanRay {
 // bin(p) = dsd (p . e_u) / ((p . e_c + dso) du) + half.
 struct FanView {
     float eux, euy, ecx, ecy, dso, dsd, du, half;
+    double deux, deuy, decx, decy, ddso, dscale, dhalf;   // the same in FP64; dscale = dsd / du
 };
 
 // Per-iteration log record (what dgamp_ct_stats exposes).
@@ -157,6 +158,7 @@ struct Workspace {
     float* b = nullptr;            // the iteration's probe b (Eq. MC_SURE) [n][n]
     FanRay* fan_rays = nullptr;    // fan-beam plans: [n_views][n_det]
     FanView* fan_views = nullptr;  // fan-beam plans: [n_views]
+    float2* fan_gw = nullptr;      // fan-beam plans whose A^T takes the pixel form: du / max(|v_x|, |v_y|), w per ray
     int* pj_order = nullptr;       // banded A: views marching over rows, then over columns [n_views]
     float* pj_part = nullptr;      // banded A: per-band partial sums [ceil(n / 16)][n_views][n_det]
 };
