@@ -174,9 +174,9 @@ __device__ __forceinline__ void img_cols_block(float2* __restrict__ C, int n, in
                                                const float2* __restrict__ tw, float f0, int inverse_gain,
                                                float2* smem) {
     const int NC = blockDim.y, kx0 = bx * NC, ms = img_stride(m), BL = fft_buf_len(m);
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * NC;
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * NC, sh = __ffs(NC) - 1;   // NC = 1, 2, 4
     for (int j = tid; j < m * NC; j += nt) {       // NC columns of a row are neighbours in memory
-        const int i = j / NC, c = j - i * NC;
+        const int i = j >> sh, c = j & (NC - 1);
         smem[2 * c * BL + fpad(i)] =
             i < n && kx0 + c <= m / 2 ? C[(size_t)i * ms + kx0 + c] : make_float2(0.f, 0.f);
     }
@@ -197,7 +197,7 @@ __device__ __forceinline__ void img_cols_block(float2* __restrict__ C, int n, in
     r = fft_stockham(r, o, m, tw, 1.f);
     const int at = (int)(r - a);                   // the same buffer of every column
     for (int j = tid; j < n * NC; j += nt) {
-        const int i = j / NC, c = j - i * NC;
+        const int i = j >> sh, c = j & (NC - 1);
         if (kx0 + c <= m / 2) C[(size_t)i * ms + kx0 + c] = smem[2 * c * BL + at + fpad(i)];
     }
 }
