@@ -262,7 +262,7 @@ k_fan_backproject_tile(const float* __restrict__ sino, const FanRay* __restrict_
 // with rel and sig linear in the pixel; q0 + rel is 6.26 fixed point from
 // FP64 constants, and only the correction -rel sig / (1 + sig), about one bin
 // at most at a scanner's proportions, is FP32.  A^T + A with both filters at
-// 512^2/102/736: 210 -> 150 us (A^T itself 124 -> about 62).
+// 512^2/102/736: 210 -> 144 us (with the tile corners in FP64 too: 150).
 constexpr int kFgS = 16, kFgThreads = 128;
 constexpr int kFgViews = 32;      // views staged at a time (16 KB)
 constexpr int kFgSlots = 64;      // rays a view can need (checked by fan_gather_ok)
@@ -292,20 +292,20 @@ __device__ __forceinline__ void fg_view_setup(const FanView* __restrict__ views,
         const double kx = k * (V.deux * s0 - t0 * V.decx), ky = -k * (V.deuy * s0 - t0 * V.decy);
         const double gx = V.decx * is0, gy = -V.decy * is0;
         const double q0 = V.dhalf + V.dscale * t0 * is0;
-        // lowest q over the tile's pixels of the image (grown by one; sig > -1 in front of the source)
-        const double xe = min(kFgS / 2, n - tx0 - kFgS / 2), ye = min(kFgS / 2, n - ty0 - kFgS / 2);
-        double ql = q0;
+        // lowest q - q0 over the tile's pixels of the image (grown by one; sig > -1 in front of the
+        // source), in FP32: only the first staged ray depends on it, and it leaves a margin
+        const float fkx = (float)kx, fky = (float)ky, fgx = (float)gx, fgy = (float)gy;
+        const float xe = (float)min(kFgS / 2, n - tx0 - kFgS / 2), ye = (float)min(kFgS / 2, n - ty0 - kFgS / 2);
+        float ql = -8.f * (fabsf(fkx) + fabsf(fky));      // the linear part may fall below q itself
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-            const double x = (h & 1) ? xe : -8.0, y = (h & 2) ? ye : -8.0;
-            ql = fmin(ql, q0 + (kx * x + ky * y) / (1.0 + gx * x + gy * y));
+            const float x = (h & 1) ? xe : -8.f, y = (h & 2) ? ye : -8.f;
+            ql = fminf(ql, (fkx * x + fky * y) / (1.f + fgx * x + fgy * y));
         }
-        // the linear part may fall below q itself: room for both, and for ray floor(q) - 1
-        ql = fmin(ql, q0 - 8.0 * (fabs(kx) + fabs(ky)));
-        const double lo = floor(ql) - 2.0;
+        const double lo = floor(q0 + ql) - 2.0;           // room for ray floor(q) - 1
         const double unit = (double)(1 << kFgFrac);
         sh.fix[i] = make_int4((int)(unsigned)((q0 - lo) * unit + 4.0), (int)rint(kx * unit), (int)rint(ky * unit), (int)lo);
-        sh.lin[i] = make_float4((float)kx, (float)ky, (float)gx, (float)gy);
+        sh.lin[i] = make_float4(fkx, fky, fgx, fgy);
         sh.s0[i] = (float)s0;
     }
 }
