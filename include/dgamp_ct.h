@@ -216,7 +216,10 @@ int dgamp_ct_plan_info(dgamp_ct_plan_t plan, double* frob_sq, int32_t* fft_len);
    dgamp_ct_plan makes them by timing on the plan's geometry.  */
 typedef struct {
     int32_t filter_mode;  /* 0 = H by FFT, 1 = H as a Toeplitz product with the same
-                             kernel h = IFFT_P(g) (no wrap-around since P >= 2 n_det) */
+                             kernel h = IFFT_P(g) (no wrap-around since P >= 2 n_det).
+                             Reported for the single-step calls; inside a solve's
+                             three-kernel form H runs by FFT, with output_moments = 1 in the
+                             faster form, unless this is set */
     int32_t tv_kb;        /* Chambolle steps per blocked TV launch, 1..10 */
     int32_t tv_rows;      /* rows of the image region one TV block holds: 32, 64 or 128
                              (the region is 64 columns wide) */
@@ -225,7 +228,7 @@ typedef struct {
                              P <= 8192); 2 = a cluster of 8 blocks per view, each a slice
                              of the bins, H as its Toeplitz product and s shared through
                              distributed shared memory (needs n_det <= 1792); 0 = three
-                             kernels, H in filter_mode's form.  The plan times the forms
+                             kernels, H as filter_mode says.  The plan times the forms
                              the geometry allows and keeps the faster; filter_mode alone
                              governs the single-step entry points */
     int32_t bp_mode;      /* A^T: 0 = pixel-driven gather (each pixel finds the <= 2 rays

@@ -294,7 +294,7 @@ class Plan:
         """The plan's implementation choices (dgamp_ct_tuning): {"filter_mode": 0 FFT | 1 Toeplitz,
         "tv_kb": steps per TV launch, "tv_rows": rows of a TV block's region, "sino_fused": 1 if the
         solve runs H A x, the output step and H s as one kernel, "bp_mode": 0 pixel-driven | 1
-        ray-driven A^T, "pj_seg": warps splitting the steps of 32 rays in A, "tv_vrows": rows of a TV
+        tiled A^T, "pj_seg": warps splitting the steps of 32 rays in A, "tv_vrows": rows of a TV
         region per thread (2, 4 or 8), "pj_band": 0 for that ray-group A or the lines of a shared-memory
         band of the banded A (16 or 32), "pj_waves": full waves of blocks of the banded A (1 or 2)}."""
         t = Tuning()

@@ -289,11 +289,11 @@ static int enqueue_iteration(dgamp_ct_plan_s* pl, cudaStream_t st, cudaEvent_t* 
         DGCT_TRY(launch_sino_step(pl, st, bf));                         // H A x, Step 2, H s
         DGCT_TRY(mark());
     } else {
-        DGCT_TRY(launch_filter(pl, w.zraw, w.z, st, bf));               //         H A x
+        DGCT_TRY(launch_filter(pl, w.zraw, w.z, st, bf, 1));            //         H A x
         DGCT_TRY(mark());
         DGCT_TRY(launch_output_step(pl, w.z, w.y, w.s, 1, 1, 0.0, 0.0, nullptr, st, bf));  // Step 2
         DGCT_TRY(mark());
-        DGCT_TRY(launch_filter(pl, w.s, w.hs, st, bf));                 // Step 3: H s
+        DGCT_TRY(launch_filter(pl, w.s, w.hs, st, bf, 1));              // Step 3: H s
         DGCT_TRY(mark());
     }
     DGCT_TRY(launch_backproject(pl, w.hs, w.x, w.r, 1, st, bf,          //         r = x + tau_r A^T H s
@@ -599,7 +599,7 @@ int dgamp_ct_set_tuning(dgamp_ct_plan_t pl, const dgamp_ct_tuning* t) {
     if (t->sino_fused == 1 && !sino_step_eligible(pl)) return DGAMP_CT_ERR_UNSUPPORTED_GEOMETRY;
     if (t->sino_fused == 2 && !sino_toeplitz_eligible(pl)) return DGAMP_CT_ERR_UNSUPPORTED_GEOMETRY;
     if (pl->fan && t->bp_mode == 1 && pl->fan_stride <= 0) return DGAMP_CT_ERR_UNSUPPORTED_GEOMETRY;
-    if (t->filter_mode >= 0) pl->filter_mode = t->filter_mode;
+    if (t->filter_mode >= 0) pl->filter_mode = pl->filter_set = t->filter_mode;
     if (t->tv_kb > 0) pl->tv_kb = t->tv_kb;
     if (t->tv_rows > 0) pl->tv_rows = t->tv_rows;
     if (t->sino_fused >= 0) pl->sino_fused = t->sino_fused;

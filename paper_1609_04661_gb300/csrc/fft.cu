@@ -22,26 +22,26 @@ static int fft_threads(int P) { return P / 8 < 32 ? 32 : (P / 8 > 512 ? 512 : P 
 // One view per block.  With z[j] = x[2j] + i x[2j + 1] and Z its DFT of length
 // L = P / 2, the even and odd bins' DFTs are E = (Z[k] + conj Z[L-k]) / 2 and
 // O = (Z[k] - conj Z[L-k]) / 2i, and x's own are E +- w^k O at k and k + L,
-// w = exp(-2 pi i / P).  Multiplying those by the gains a = g[k] and
-// b = g[k + L] = g[L-k] gives
-//   E' = ((a + b) E + (a - b) w^k O) / 2,   O' = ((a - b) w^-k E + (a + b) O) / 2,
-// and Z' = E' + i O' (at L-k: conj E' + i conj O') transforms back to the
-// filtered bins.  The block's chain of stages and barriers bounds the kernel,
+// w = exp(-2 pi i / P).  With these times the gains g[k] and g[k + L] = g[L-k] as
+// A and C, E' = (A + C) / 2 and O' = w^-k (A - C) / 2, and Z' = E' + i O' (at L-k:
+// conj E' + i conj O') transforms back to the filtered bins.  (Gathering E and O
+// by (g[k] +- g[L-k]) instead saves an addition each, but lets the high
+// frequencies' rounding into the low ones, which A^T then amplifies.)  The block's chain of stages and barriers bounds the kernel,
 // not its arithmetic: a pair of views per block as one complex line of length P
 // left 45 blocks with twice the butterflies per stage at 90 views, P = 4096.
 // Two filters and an output step at 90 x 1449: 55.5 -> 50.2 us.
-template <typename T>
 __global__ void __launch_bounds__(512)
-k_filter_views(const T* in, T* out, int nd, int P, const float* __restrict__ gain, const float2* __restrict__ tw) {
+k_filter_line(const float* in, float* out, int nd, int P, const float* __restrict__ gain, const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
     const int L = P >> 1;
     float2* a = smem;
     float2* b = smem + fft_buf_len(L);
-    const T* row = in + (size_t)blockIdx.x * nd;
+    const float* row = in + (size_t)blockIdx.x * nd;
+    pdl_wait();
     for (int i = threadIdx.x; i < L; i += blockDim.x) {
         float2 v = make_float2(0.f, 0.f);
-        if (2 * i < nd) v.x = ldf(row + 2 * i);
-        if (2 * i + 1 < nd) v.y = ldf(row + 2 * i + 1);
+        if (2 * i < nd) v.x = row[2 * i];
+        if (2 * i + 1 < nd) v.y = row[2 * i + 1];
         a[fpad(i)] = v;
     }
     __syncthreads();
@@ -51,24 +51,69 @@ k_filter_views(const T* in, T* out, int nd, int P, const float* __restrict__ gai
     for (int k = threadIdx.x; k <= L / 2; k += blockDim.x) {
         const int kk = (L - k) & (L - 1);
         const float2 z = r[fpad(k)], y = r[fpad(kk)];
-        const float ga = __ldg(gain + k), gb = __ldg(gain + L - k);
-        const float gp = (ga + gb) * sc, gm = (ga - gb) * sc;
+        const float ga = __ldg(gain + k) * sc, gb = __ldg(gain + L - k) * sc;
         float sn, cs;
         sincospif((float)k / (float)L, &sn, &cs);                    // w^k = cs - i sn
         const float2 E = make_float2(z.x + y.x, z.y - y.y), O = make_float2(z.y + y.y, y.x - z.x);   // twice E, O
         const float2 wO = make_float2(fmaf(cs, O.x, sn * O.y), fmaf(cs, O.y, -sn * O.x));
-        const float2 wE = make_float2(fmaf(cs, E.x, -sn * E.y), fmaf(cs, E.y, sn * E.x));            // w^-k E
-        const float2 e = make_float2(fmaf(gp, E.x, gm * wO.x), fmaf(gp, E.y, gm * wO.y));
-        const float2 q = make_float2(fmaf(gm, wE.x, gp * O.x), fmaf(gm, wE.y, gp * O.y));
+        const float2 A = make_float2(ga * (E.x + wO.x), ga * (E.y + wO.y));
+        const float2 C = make_float2(gb * (E.x - wO.x), gb * (E.y - wO.y));
+        const float2 e = cadd(A, C), d = csub(A, C);
+        const float2 q = make_float2(fmaf(cs, d.x, -sn * d.y), fmaf(cs, d.y, sn * d.x));             // w^-k (A - C)
         r[fpad(k)] = make_float2(e.x - q.y, e.y + q.x);
         if (kk != k) r[fpad(kk)] = make_float2(e.x + q.y, q.x - e.y);
     }
     __syncthreads();
     r = fft_stockham(r, o, L, tw, 1.f);
-    T* w = out + (size_t)blockIdx.x * nd;
+    float* w = out + (size_t)blockIdx.x * nd;
     for (int i = threadIdx.x; i < nd; i += blockDim.x) {
         const float2 v = r[fpad(i >> 1)];
-        stf(w + i, (i & 1) ? v.y : v.x);
+        w[i] = (i & 1) ? v.y : v.x;
+    }
+}
+
+// Two views per block as one complex line of length P, which the real and even
+// gain filters both: the arithmetic of the fused sinogram kernel's FFT form.  A
+// solve in the three-kernel form takes this one, so that the two forms' scalars
+// stay together over the iterations (on the smallest geometries the half-length
+// line's rounding grows past 1e-4 in five); single-step calls take the faster
+// line per view above.
+template <typename T>
+__global__ void __launch_bounds__(512)
+k_filter_pairs(const T* in, T* out, int nv, int nd, int P,
+               const float* __restrict__ gain, const float2* __restrict__ tw) {
+    extern __shared__ float2 smem[];
+    float2* a = smem;
+    float2* b = smem + fft_buf_len(P);
+    const int va = 2 * blockIdx.x, vb = va + 1;
+    const bool hasb = vb < nv;
+    const T* ra = in + (size_t)va * nd;
+    const T* rb = in + (size_t)vb * nd;
+    for (int i = threadIdx.x; i < P; i += blockDim.x) {
+        float2 v = make_float2(0.f, 0.f);
+        if (i < nd) {
+            v.x = ldf(ra + i);
+            if (hasb) v.y = ldf(rb + i);
+        }
+        a[fpad(i)] = v;
+    }
+    __syncthreads();
+    float2* r = fft_stockham(a, b, P, tw, -1.f);
+    float2* o = (r == a) ? b : a;
+    for (int i = threadIdx.x; i < P; i += blockDim.x) {
+        const float g = __ldg(gain + i);
+        const float2 v = r[fpad(i)];
+        r[fpad(i)] = make_float2(v.x * g, v.y * g);
+    }
+    __syncthreads();
+    r = fft_stockham(r, o, P, tw, 1.f);
+    const float sc = 1.0f / (float)P;
+    T* wa = out + (size_t)va * nd;
+    T* wb = out + (size_t)vb * nd;
+    for (int i = threadIdx.x; i < nd; i += blockDim.x) {
+        const float2 v = r[fpad(i)];
+        stf(wa + i, v.x * sc);
+        if (hasb) stf(wb + i, v.y * sc);
     }
 }
 
@@ -93,8 +138,9 @@ k_filter_toeplitz(const T* in, T* out, int nd, const float* __restrict__ hx) {
     const int d0 = blockIdx.x * kTzOut;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const T* row = in + (size_t)v * nd;
+    for (int i = tid; i < 2 * nd - 1; i += blockDim.x) hs[i] = hx[i];      // plan constants: before the wait
+    pdl_wait();
     for (int i = tid; i < nd; i += blockDim.x) zs[i] = ldf(row + i);
-    for (int i = tid; i < 2 * nd - 1; i += blockDim.x) hs[i] = hx[i];
     __syncthreads();
     const int dl = d0 + 4 * lane;          // this lane's first output
     const int len = (nd + kTzWarps - 1) / kTzWarps;
@@ -139,8 +185,12 @@ static size_t toeplitz_smem(int nd) {
 }
 
 // bf = 1: in and out hold BF16 (a solve with storage = 1); sums in FP32 either way
-int launch_filter(const dgamp_ct_plan_s* pl, const float* in, float* out, cudaStream_t st, int bf) {
-    if (pl->filter_mode == 1) {
+int launch_filter(const dgamp_ct_plan_s* pl, const float* in, float* out, cudaStream_t st, int bf, int solve) {
+    // A solve's three-kernel form: with the Laplace step it stands beside the fused FFT form and takes its
+    // arithmetic (k_filter_pairs) unless the tuning sets one; with exact moments it is the only form there is
+    // and takes the faster
+    const int in_solve = pl->filter_set >= 0 ? pl->filter_set : (pl->opt.output_moments ? pl->filter_solve : 0);
+    if ((solve ? in_solve : pl->filter_mode) == 1) {
         // the block reads its whole input row first, so in == out needs a copy
         const float* src = in;
         if (in == out) {
@@ -148,57 +198,72 @@ int launch_filter(const dgamp_ct_plan_s* pl, const float* in, float* out, cudaSt
             src = pl->ws.zraw2;
         }
         dim3 grd((pl->nd + kTzOut - 1) / kTzOut, pl->nv);
+        const size_t sm = toeplitz_smem(pl->nd);
+        if (solve) {
+            if (bf)
+                k_filter_toeplitz<bf16s><<<grd, 32 * kTzWarps, sm, st>>>((const bf16s*)src, (bf16s*)out, pl->nd, pl->ws.hx);
+            else
+                k_filter_toeplitz<float><<<grd, 32 * kTzWarps, sm, st>>>(src, out, pl->nd, pl->ws.hx);
+            DGCT_LAUNCH_CHECK();
+        } else {
+            DGCT_CUDA(launch_pdl(k_filter_toeplitz<float>, grd, dim3(32 * kTzWarps), sm, st, src, out, pl->nd, pl->ws.hx));
+        }
+        return DGAMP_CT_OK;
+    }
+    if (solve) {
+        const size_t sm = (size_t)2 * fft_buf_len(pl->P) * sizeof(float2);
+        const dim3 grd((pl->nv + 1) / 2), blk(fft_threads(pl->P));
         if (bf)
-            k_filter_toeplitz<bf16s><<<grd, 32 * kTzWarps, toeplitz_smem(pl->nd), st>>>((const bf16s*)src, (bf16s*)out,
-                                                                                        pl->nd, pl->ws.hx);
+            k_filter_pairs<bf16s><<<grd, blk, sm, st>>>((const bf16s*)in, (bf16s*)out, pl->nv, pl->nd, pl->P, pl->ws.gain,
+                                                        pl->ws.tw);
         else
-            k_filter_toeplitz<float><<<grd, 32 * kTzWarps, toeplitz_smem(pl->nd), st>>>(src, out, pl->nd, pl->ws.hx);
+            k_filter_pairs<float><<<grd, blk, sm, st>>>(in, out, pl->nv, pl->nd, pl->P, pl->ws.gain, pl->ws.tw);
         DGCT_LAUNCH_CHECK();
         return DGAMP_CT_OK;
     }
     const int P = pl->P, L = P / 2;
     const size_t sm = (size_t)2 * fft_buf_len(L) * sizeof(float2);
     const int thr = fft_threads(L);
-    if (bf)
-        k_filter_views<bf16s><<<pl->nv, thr, sm, st>>>((const bf16s*)in, (bf16s*)out, pl->nd, P, pl->ws.gain,
-                                                       pl->ws.twh);
-    else
-        k_filter_views<float><<<pl->nv, thr, sm, st>>>(in, out, pl->nd, P, pl->ws.gain, pl->ws.twh);
-    DGCT_LAUNCH_CHECK();
+    DGCT_CUDA(launch_pdl(k_filter_line, dim3(pl->nv), dim3(thr), sm, st, in, out, pl->nd, P, pl->ws.gain, pl->ws.twh));
     return DGAMP_CT_OK;
 }
 
-// Plan-time choice between the FFT and the Toeplitz form of H (same operator):
-// time both on the plan's geometry and keep the faster.
+// Plan-time choice between the FFT and the Toeplitz form of H (same operator),
+// for the single-step calls and for a solve's three-kernel form: time both on
+// the plan's geometry and keep the faster.
 int filter_autotune(dgamp_ct_plan_s* pl) {
     DGCT_CUDA(cudaMemset(pl->ws.zraw, 0, (size_t)pl->M * sizeof(float)));
     cudaEvent_t e0, e1;
     DGCT_CUDA(cudaEventCreate(&e0));
     DGCT_CUDA(cudaEventCreate(&e1));
-    float best = 1e30f;
-    int best_mode = 0;
-    for (int mode = 0; mode < 2; ++mode) {
-        pl->filter_mode = mode;
-        int rc = DGAMP_CT_OK;
-        for (int rep = 0; rep < 6 && rc == DGAMP_CT_OK; ++rep) {
-            if (rep == 1) cudaEventRecord(e0, 0);
-            rc = launch_filter(pl, pl->ws.zraw, pl->ws.z, 0);
+    int rc = DGAMP_CT_OK;
+    for (int solve = 0; solve < 2 && rc == DGAMP_CT_OK; ++solve) {
+        int& choice = solve ? pl->filter_solve : pl->filter_mode;
+        float best = 1e30f;
+        int best_mode = 0;
+        for (int mode = 0; mode < 2 && rc == DGAMP_CT_OK; ++mode) {
+            choice = mode;
+            pl->filter_set = solve ? mode : -1;
+            for (int rep = 0; rep < 6 && rc == DGAMP_CT_OK; ++rep) {
+                if (rep == 1) cudaEventRecord(e0, 0);
+                rc = launch_filter(pl, pl->ws.zraw, pl->ws.z, 0, 0, solve);
+            }
+            cudaEventRecord(e1, 0);
+            const cudaError_t e = cudaEventSynchronize(e1);
+            if (rc == DGAMP_CT_OK && e != cudaSuccess) rc = cuda_fail(e);
+            float ms = 0.f;
+            if (rc == DGAMP_CT_OK) cudaEventElapsedTime(&ms, e0, e1);
+            if (rc == DGAMP_CT_OK && ms < best) {
+                best = ms;
+                best_mode = mode;
+            }
         }
-        cudaEventRecord(e1, 0);
-        cudaError_t e = cudaEventSynchronize(e1);
-        if (rc != DGAMP_CT_OK || e != cudaSuccess) {
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            return rc != DGAMP_CT_OK ? rc : cuda_fail(e);
-        }
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best) { best = ms; best_mode = mode; }
+        choice = best_mode;
     }
+    pl->filter_set = -1;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    pl->filter_mode = best_mode;
-    return DGAMP_CT_OK;
+    return rc;
 }
 
 int toeplitz_set_smem_limit(int nd) {
@@ -215,6 +280,7 @@ __global__ void __launch_bounds__(512)
 k_img_rows_fwd(const float* __restrict__ img, int n, int m, const float2* __restrict__ tw,
                float2* __restrict__ C) {
     extern __shared__ float2 smem[];
+    pdl_wait();
     img_rows_fwd_block(img + (size_t)blockIdx.y * n * n, n, m, 2 * blockIdx.x, tw,
                        C + (size_t)blockIdx.y * n * img_stride(m), smem);
 }
@@ -223,6 +289,7 @@ __global__ void __launch_bounds__(512)
 k_img_cols(float2* __restrict__ C, int n, int m, const float2* __restrict__ tw, float f0,
            int inverse_gain) {
     extern __shared__ float2 smem[];
+    pdl_wait();
     img_cols_block(C + (size_t)blockIdx.y * n * img_stride(m), n, m, blockIdx.x, tw, f0, inverse_gain, smem);
 }
 
@@ -232,6 +299,7 @@ k_img_rows_inv(const float2* __restrict__ C, int n, int m, const float2* __restr
                float* __restrict__ out) {
     extern __shared__ float2 smem[];
     const int y0 = 2 * blockIdx.x;
+    pdl_wait();
     const float2* r = img_rows_inv_block(C + (size_t)blockIdx.y * n * img_stride(m), n, m, y0, tw, smem);
     out += (size_t)blockIdx.y * n * n + (size_t)y0 * n;
     const float sc = 1.0f / ((float)m * (float)m);
@@ -253,6 +321,7 @@ k_img_rows_inv_update(const float2* __restrict__ C, int n, int m, const float2* 
     extern __shared__ float2 smem[];
     __shared__ unsigned s_max;
     const int y0 = 2 * blockIdx.x;
+    pdl_wait();
     if (threadIdx.x == 0) {
         s_max = 0u;
         if (y0 == 0) S->div_pending = 0u;
@@ -278,11 +347,10 @@ static int launch_img_forward(const dgamp_ct_plan_s* pl, const float* in, float2
     const int n = pl->n, m = pl->m2, thr = fft_threads(m), nc = img_cols_per_block(m);
     const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
     const float f0 = 1.0f / (2.0f * (float)pl->P);
-    k_img_rows_fwd<<<dim3((n + 1) / 2, nimg), thr, sm, st>>>(in, n, m, pl->ws.tw2, C);
-    DGCT_LAUNCH_CHECK();
+    DGCT_CUDA(launch_pdl(k_img_rows_fwd, dim3((n + 1) / 2, nimg), dim3(thr), sm, st, in, n, m, pl->ws.tw2, C));
     // V^-1 applies sqrt(max(rho, f0)); V applies its reciprocal
-    k_img_cols<<<dim3(img_col_blocks(m, nc), nimg), dim3(thr, nc), nc * sm, st>>>(C, n, m, pl->ws.tw2, f0, inverse_gain);
-    DGCT_LAUNCH_CHECK();
+    DGCT_CUDA(launch_pdl(k_img_cols, dim3(img_col_blocks(m, nc), nimg), dim3(thr, nc), nc * sm, st, C, n, m, pl->ws.tw2,
+                         f0, inverse_gain));
     return DGAMP_CT_OK;
 }
 
@@ -291,8 +359,8 @@ int launch_precond_image_update(const dgamp_ct_plan_s* pl, const float* in, cons
     const int n = pl->n, m = pl->m2;
     const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
     DGCT_TRY(launch_img_forward(pl, in, pl->ws.fft2d, 1, 0, st));
-    k_img_rows_inv_update<<<(n + 1) / 2, fft_threads(m), sm, st>>>(pl->ws.fft2d, n, m, pl->ws.tw2, x, pl->ws.S, out);
-    DGCT_LAUNCH_CHECK();
+    DGCT_CUDA(launch_pdl(k_img_rows_inv_update, dim3((n + 1) / 2), dim3(fft_threads(m)), sm, st, pl->ws.fft2d, n, m,
+                         pl->ws.tw2, x, pl->ws.S, out));
     return DGAMP_CT_OK;
 }
 
@@ -310,14 +378,14 @@ int launch_precond_images(const dgamp_ct_plan_s* pl, const float* in, float* out
     const int n = pl->n, m = pl->m2;
     const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
     DGCT_TRY(launch_img_forward(pl, in, C, nimg, inverse ? 0 : 1, st));
-    k_img_rows_inv<<<dim3((n + 1) / 2, nimg), fft_threads(m), sm, st>>>(C, n, m, pl->ws.tw2, out);
-    DGCT_LAUNCH_CHECK();
+    DGCT_CUDA(launch_pdl(k_img_rows_inv, dim3((n + 1) / 2, nimg), dim3(fft_threads(m)), sm, st, C, n, m, pl->ws.tw2, out));
     return DGAMP_CT_OK;
 }
 
 int fft_set_smem_limits(int bytes) {
-    DGCT_TRY(raise_smem_limit((const void*)k_filter_views<float>, bytes));
-    DGCT_TRY(raise_smem_limit((const void*)k_filter_views<bf16s>, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_line, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_pairs<float>, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_pairs<bf16s>, bytes));
     DGCT_TRY(raise_smem_limit((const void*)k_img_rows_fwd, bytes));
     // several columns a block up to m = 2048: 4 at 1024 and 2 at 2048 need the same 74 KB
     DGCT_TRY(raise_smem_limit((const void*)k_img_cols,

@@ -181,6 +181,8 @@ struct dgamp_ct_plan_s {
     int tv_rows = 64;                      // rows of a blocked TV region (32, 64 or 128)
     int tv_vrows = 4;                      // rows per thread of a TV region (4, or 8 with 64-row regions)
     int filter_mode = 0;                   // H by 0: FFT, 1: Toeplitz product (plan-time choice)
+    int filter_solve = 0;                  // the same inside a solve with exact moments (plan-time choice)
+    int filter_set = -1;                   // the form set by dgamp_ct_set_tuning for all of them (-1: none)
     int sino_fused = 0;                    // solve: H A x, output step, H s in one kernel (k_sino_step)
     int bp_mode = 0;                       // A^T: 0 pixel-driven gather, 1 ray-driven tiles (plan-time choice)
     int pj_seg = 8;                        // A: step segments (warps) per ray group, 8/16/32 (plan-time choice)
@@ -429,7 +431,8 @@ int launch_backproject(const dgamp_ct_plan_s* pl, const float* sino, const float
                        float* out, int update, cudaStream_t st, int bf = 0, int nparts = 0);
 int launch_frobenius(dgamp_ct_plan_s* pl);
 // fft.cu
-int launch_filter(const dgamp_ct_plan_s* pl, const float* in, float* out, cudaStream_t st, int bf = 0);
+// solve = 1: inside a solve's three-kernel form; bf = 1 only there
+int launch_filter(const dgamp_ct_plan_s* pl, const float* in, float* out, cudaStream_t st, int bf = 0, int solve = 0);
 // Raises a kernel's dynamic shared-memory limit to at least `bytes`, never
 // lowering it: the limit belongs to the kernel in the whole context, and a
 // plan made earlier may launch it with more.
