@@ -75,8 +75,10 @@ k_fan_project(const T* __restrict__ XR, const T* __restrict__ XC, int ldp, int n
     const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
     const int d = blockIdx.x * 32 + lane;
     float acc = 0.f, w = 0.f;
+    FanRay R{};
+    if (d < nd) R = rays[(size_t)v * nd + d];      // plan constants: before the wait
+    pdl_wait();      // the staged image is the previous kernel's output
     if (d < nd) {
-        const FanRay R = rays[(size_t)v * nd + d];
         w = R.w;
         const T* __restrict__ B = R.col ? XC : XR;
         int s0, s1;
@@ -391,6 +393,7 @@ k_fan_backproject_gather(const float* __restrict__ sino, const float2* __restric
         const int cnt = min(kFgViews, nv - v0);
         if (v0 > 0) __syncthreads();                                       // the previous views are done with
         fg_view_setup(views, v0, cnt, n, tx0, ty0, sh);
+        if (v0 == 0) pdl_wait();      // the views are plan constants, the sinogram is not
         __syncthreads();
         const bool bad = fg_stage(sino, gw, v0, cnt, nd, sh);
         if (__syncthreads_or(bad))
@@ -516,17 +519,16 @@ static void fan_constants(int n, int nd, const std::vector<double>& ang, double 
 
 int launch_fan_project(const dgamp_ct_plan_s* pl, float* sino, cudaStream_t st) {
     const dim3 grd((unsigned)((pl->nd + 31) / 32), (unsigned)pl->nv);
-    k_fan_project<float><<<grd, 32 * kFanSeg, 0, st>>>(pl->ws.XR, pl->ws.XC, pl->ldp, pl->n, pl->nd,
-                                                       pl->ws.fan_rays, sino);
-    DGCT_LAUNCH_CHECK();
+    DGCT_CUDA(launch_pdl(k_fan_project<float>, grd, dim3(32 * kFanSeg), 0, st, pl->ws.XR, pl->ws.XC, pl->ldp, pl->n,
+                         pl->nd, pl->ws.fan_rays, sino));
     return DGAMP_CT_OK;
 }
 
 int launch_fan_backproject(const dgamp_ct_plan_s* pl, const float* sino, float* img, cudaStream_t st) {
     const dim3 grd((unsigned)((pl->n + 15) / 16), (unsigned)((pl->n + 15) / 16));
     if (pl->bp_mode == 1 && pl->fan_stride > 0 && pl->ws.fan_gw)
-        k_fan_backproject_gather<<<grd, kFgThreads, 0, st>>>(sino, pl->ws.fan_gw, pl->ws.fan_views, pl->n, pl->nv,
-                                                             pl->nd, img);
+        DGCT_CUDA(launch_pdl(k_fan_backproject_gather, grd, dim3(kFgThreads), 0, st, sino, pl->ws.fan_gw,
+                             pl->ws.fan_views, pl->n, pl->nv, pl->nd, img));
     else if (pl->bp_mode == 1 && pl->fan_stride > 0)
         k_fan_backproject_tile<<<grd, kFtWarps * 32, 0, st>>>(sino, pl->ws.fan_rays, pl->ws.fan_views, pl->n, pl->nv,
                                                               pl->nd, pl->fan_stride, img);

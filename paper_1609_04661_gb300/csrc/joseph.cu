@@ -19,6 +19,7 @@ __global__ void k_stage_image(const float* __restrict__ img, int n, int ldp,
                               T* __restrict__ XR, T* __restrict__ XC) {
     __shared__ float tile[32][33];
     const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
+    pdl_wait();
     for (int j = threadIdx.y; j < 32; j += blockDim.y) {
         const int iy = by + j, ix = bx + threadIdx.x;
         float v = 0.f;
@@ -53,10 +54,10 @@ __global__ void k_stage_image(const float* __restrict__ img, int n, int ldp,
 int launch_stage_image(const dgamp_ct_plan_s* pl, const float* img, cudaStream_t st, int bf) {
     dim3 blk(32, 8), grd((pl->n + 31) / 32, (pl->n + 31) / 32);
     if (bf)
-        k_stage_image<bf16s><<<grd, blk, 0, st>>>(img, pl->n, pl->ldp, (bf16s*)pl->ws.XR, (bf16s*)pl->ws.XC);
+        DGCT_CUDA(launch_pdl(k_stage_image<bf16s>, grd, blk, 0, st, img, pl->n, pl->ldp, (bf16s*)pl->ws.XR,
+                             (bf16s*)pl->ws.XC));
     else
-        k_stage_image<float><<<grd, blk, 0, st>>>(img, pl->n, pl->ldp, pl->ws.XR, pl->ws.XC);
-    DGCT_LAUNCH_CHECK();
+        DGCT_CUDA(launch_pdl(k_stage_image<float>, grd, blk, 0, st, img, pl->n, pl->ldp, pl->ws.XR, pl->ws.XC));
     return DGAMP_CT_OK;
 }
 

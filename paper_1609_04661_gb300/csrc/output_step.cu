@@ -13,6 +13,7 @@ k_output_step(const T* z, const float* y, T* s, long long M, int use_prev,
               const double* partial_div, double floor_rel, IterLog* log, int exact) {
     __shared__ double sm[32];
     __shared__ float s_tp, s_inv, s_logI0;
+    pdl_wait();
     if (threadIdx.x < 32) {
         const double tx = from_scalars ? pending_tau_x(S, partial_div, N, floor_rel, log, blockIdx.x == 0) : 0.0;
         if (threadIdx.x == 0) {
@@ -48,17 +49,15 @@ int launch_output_step(const dgamp_ct_plan_s* pl, const float* z, const float* y
     const int onsager = from_scalars ? pl->opt.onsager : 1;
     const float damp_s = from_scalars ? (float)pl->opt.damp_s : 1.f;
     if (bf)   // z and s in BF16 (a solve with storage = 1); the counts stay FP32
-        k_output_step<bf16s><<<blocks, 128, 0, st>>>((const bf16s*)z, y, (bf16s*)s, M, use_prev, from_scalars,
-                                                     tau_p_arg, logI0_arg, onsager, damp_s, pl->opt.truncate_z,
-                                                     (double)pl->N, pl->ws.S, pl->ws.partial, tau_s_out,
-                                                     pl->ws.partial_div, pl->opt.tau_x_floor, pl->ws.log,
-                                                     pl->opt.output_moments);
+        DGCT_CUDA(launch_pdl(k_output_step<bf16s>, dim3(blocks), dim3(128), 0, st, (const bf16s*)z, y, (bf16s*)s, M,
+                             use_prev, from_scalars, tau_p_arg, logI0_arg, onsager, damp_s, pl->opt.truncate_z,
+                             (double)pl->N, pl->ws.S, pl->ws.partial, tau_s_out, pl->ws.partial_div,
+                             pl->opt.tau_x_floor, pl->ws.log, pl->opt.output_moments));
     else
-        k_output_step<float><<<blocks, 128, 0, st>>>(z, y, s, M, use_prev, from_scalars, tau_p_arg, logI0_arg,
-                                                     onsager, damp_s, pl->opt.truncate_z, (double)pl->N, pl->ws.S,
-                                                     pl->ws.partial, tau_s_out, pl->ws.partial_div,
-                                                     pl->opt.tau_x_floor, pl->ws.log, pl->opt.output_moments);
-    DGCT_LAUNCH_CHECK();
+        DGCT_CUDA(launch_pdl(k_output_step<float>, dim3(blocks), dim3(128), 0, st, z, y, s, M, use_prev, from_scalars,
+                             tau_p_arg, logI0_arg, onsager, damp_s, pl->opt.truncate_z, (double)pl->N, pl->ws.S,
+                             pl->ws.partial, tau_s_out, pl->ws.partial_div, pl->opt.tau_x_floor, pl->ws.log,
+                             pl->opt.output_moments));
     return DGAMP_CT_OK;
 }
 
