@@ -210,7 +210,7 @@ def _training(dg, steps: int = 20):
     return {"workload": f"17-layer 64-channel network, {B} patches of {H}x{W}, Adam, loss read back each step",
             "ms_per_step": ms, "patches_per_s": B / (ms * 1e-3), "flop_per_step": flop,
             "tflops": achieved, "frac_of_bf16_peak": achieved / peak, "peak_kind": f"{kind} cuBLAS bf16 burst",
-            "note": "64-wide patches fill half of each 128-pixel strip of the tensor-core kernels"}
+            "note": "64-wide patches go two images to a 128-pixel strip of the tensor-core convolutions"}
 
 
 def _ablation(plan, case, counts, T):
