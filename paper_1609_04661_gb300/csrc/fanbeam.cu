@@ -270,6 +270,7 @@ constexpr int kFgViews = 32;      // views staged at a time (16 KB)
 constexpr int kFgSlots = 64;      // rays a view can need (checked by fan_gather_ok)
 constexpr int kFgUnroll = 8, kFgBatch = 4;
 constexpr int kFgFrac = 26;
+constexpr double kFgMaxStep = 3.0;   // widest ray spacing in pixels (fan_gather_ok)
 
 struct FgShared {
     float2 seg[kFgViews][kFgSlots];       // A_d / s, w_d v_d
@@ -306,7 +307,7 @@ __device__ __forceinline__ void fg_view_setup(const FanView* __restrict__ views,
         }
         const double lo = floor(q0 + ql) - 2.0;           // room for ray floor(q) - 1
         const double unit = (double)(1 << kFgFrac);
-        sh.fix[i] = make_int4((int)(unsigned)((q0 - lo) * unit + 4.0), (int)rint(kx * unit), (int)rint(ky * unit), (int)lo);
+        sh.fix[i] = make_int4((int)(unsigned)((q0 - lo) * unit + 0.5), (int)rint(kx * unit), (int)rint(ky * unit), (int)lo);
         sh.lin[i] = make_float4(fkx, fky, fgx, fgy);
         sh.s0[i] = (float)s0;
     }
@@ -348,8 +349,8 @@ template <bool SAFE>
 __device__ __forceinline__ void fg_pixel(const float2* __restrict__ seg, unsigned q, float rel, float sig, float s0,
                                          float& acc) {
     const float corr = -__fdividef(rel * sig, 1.f + sig);
-    const float f = __uint_as_float(0x3F800000u | ((q >> (kFgFrac - 23)) & 0x7FFFFFu)) - 1.f;
-    const float g = f + corr, r = (g - 0.5f) + 12582912.f;          // floor(g), up to a tie
+    const float f = __uint2float_rn(q & ((1u << kFgFrac) - 1u));
+    const float g = fmaf(f, 1.f / (float)(1 << kFgFrac), corr), r = (g - 0.5f) + 12582912.f;     // floor(g), up to a tie
     const int base = min(max((int)(q >> kFgFrac) + (__float_as_int(r) - 0x4B400000), 1), kFgSlots - 3);
     const float u = g - (r - 12582912.f), s = fmaf(s0, sig, s0);
 #pragma unroll
@@ -363,6 +364,7 @@ __device__ __forceinline__ void fg_pixel(const float2* __restrict__ seg, unsigne
 template <bool SAFE>
 __device__ __forceinline__ void fg_views(const FgShared& sh, int cnt, int lx, int ly, float& acc0, float& acc1) {
     const float fx = (float)lx, fy = (float)ly;
+    float g0 = 0.f, g1 = 0.f;      // a chunk's views apart from the pixel's sum: shorter chains of additions
     for (int i0 = 0; i0 < cnt; i0 += kFgUnroll) {
         float t0 = 0.f, t1 = 0.f;
 #pragma unroll
@@ -376,9 +378,11 @@ __device__ __forceinline__ void fg_views(const FgShared& sh, int cnt, int lx, in
             fg_pixel<SAFE>(sh.seg[i], q, rel, sig, s0, t0);
             fg_pixel<SAFE>(sh.seg[i], q + 8u * (unsigned)c.z, fmaf(8.f, l.y, rel), fmaf(8.f, l.w, sig), s0, t1);
         }
-        acc0 += t0;
-        acc1 += t1;
+        g0 += t0;
+        g1 += t1;
     }
+    acc0 += g0;
+    acc1 += g1;
 }
 
 __global__ void __launch_bounds__(kFgThreads, 8)
@@ -406,14 +410,19 @@ k_fan_backproject_gather(const float* __restrict__ sino, const float2* __restric
     if (ix < n && iy + 8 < n) img[(size_t)(iy + 8) * n + ix] = acc1;
 }
 
-// Whether the pixel form applies: at the shallowest depth of the image's
-// circumscribed circle rays are at least half a pixel apart along any ray's
-// axis, and a tile's rays fit the staged slots.  q's gradient is
+// Whether the pixel form applies: inside the image's circumscribed circle rays
+// are between 1/2 and kFgMaxStep pixels apart along any ray's axis, and a tile's
+// rays fit the staged slots.  A position's rounding, a fixed share of a bin, grows
+// with the spacing in pixels: against 64 bits A^T s was off by 0.85 times as much
+// as from the ray-driven tiles at spacings up to 2.7, 0.91 at 3.2, but 1.04-1.2 at
+// 4.2, 2 at 8.5 and 17 at 68 (2.4e-6), so wider rays keep those.  q's gradient is
 // (dsd / du) sqrt(s^2 + t^2) / s^2 (t = p . e_u); its largest value is taken over the
 // circle grown to hold the centre pixel of a tile that the image's edge cuts.
 static bool fan_gather_ok(int n, double dso, double ddo, double du, int nd) {
     const double dsd = dso + ddo, u = 0.5 * (nd - 1) * du, R = n / std::sqrt(2.0) + 1.0, Rc = R + 12.0;
     if (!(dso - Rc >= 1.0) || !(du * (dso - R) / std::hypot(dsd, u) >= 0.5)) return false;
+    // max(|v_x|, |v_y|) >= |v| / sqrt 2 >= dsd / sqrt 2
+    if (!(du * (dso + R) * std::sqrt(2.0) / dsd <= kFgMaxStep)) return false;
     double grad = 0.0;
     for (int k = 0; k <= 1024; ++k) {
         const double a = 3.14159265358979 * k / 1024, s = dso - Rc * std::cos(a), t = Rc * std::sin(a);
