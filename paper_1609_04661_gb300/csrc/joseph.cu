@@ -435,57 +435,73 @@ k_backproject(const T* __restrict__ sino, int nv, int nd, int n,
 //
 // Positions are 5.27 fixed point relative to the tile: the tile's detector
 // coordinate comes from the view's 64-bit constants (units of 2^-40 bins), so
-// only the offsets inside the tile round (8 pixels at 2^-28 each).  The weights
-// then lie within 2^-22 of the projector's, which truncates its fraction to
-// 23 bits.  Rays of the views are staged kBtViews views at a time as pairs
-// (v[d] w, v[d + 1] w); a lane reads 16 consecutive pixels' pairs, at most
-// one apart, without bank conflicts.  Views are summed in order, in partial
-// sums of kBtUnroll, by one thread per pixel pair, so the result does not
-// depend on scheduling.  Per iteration of the 512^2/64/729 solve about 30.7 ->
-// 16 us; one call at 1024^2/90/1449 124 -> about 59 us.  What is left is issue
-// (half of the cycles) and the set-up and staging of blocks that all start at
-// once.  8 blocks per SM: 10 spill, 6 are slower.
+// only the offsets inside the tile round (8 pixels at 2^-28 each).  The fraction
+// is converted whole and the weights are 1 - A f and (1 - A) + A f, exact but for
+// A's own rounding and the FMA's (from a mantissa f in [1, 2) the constants were
+// 1 + A and 1 - 2 A, multiples of 2^-22 and 2^-23, which A^T s showed): within
+// 2^-22 of the projector's, which truncates its fraction to 23 bits.  Rays of the
+// views are staged kBtViews views at a time as pairs (v[d] w, v[d + 1] w); a lane
+// reads 16 consecutive pixels' pairs, at most one apart, without bank conflicts.
+// One thread per pixel pair sums the views in a fixed order -- kBtUnroll spread
+// over the chunk's angles, then four such sums, then those -- so the result does
+// not depend on scheduling.  Against 64 bits A^T s is off by 0.87 times what the
+// accumulator tiles gave (24 geometries of 64^2 .. 1024^2, 0.74 .. 0.97; 1.01 with
+// the views in sequence, 1.2 with the mantissa's weights and one chain of sums).
+// Per iteration of the 512^2/64/729 solve about 30.7 -> 16 us; one call at
+// 1024^2/90/1449 124 -> about 59 us, of which the order of the views takes 1.
+// What is left is issue (half of the cycles) and the set-up and staging of blocks
+// that all start at once.  8 blocks per SM: 10 spill, 6 are slower.
 constexpr int kBtS = 16;
 constexpr int kBtWork = 128;                  // threads that take pixels (two each)
 constexpr int kBtThreads = kBtWork + 32;      // and a warp that forms tau_r meanwhile
 constexpr int kBtViews = 64;     // views staged at a time (16 KB)
 constexpr int kBtSlots = 32;     // ray pairs a view can need: 16 (|cos| + |sin|) + 3 < 27
 constexpr int kBtUnroll = 8;
+constexpr int kBtGroup = 32;     // views whose partial sums of kBtUnroll are added before they join the pixel's sum
 constexpr int kBtFrac = 27;      // fraction bits of a tile-relative position
 constexpr int kQFrac = 40;       // fraction bits of ViewConst's Q0, QX, QY
 
 struct BtShared {
     float2 seg[kBtViews][kBtSlots];
-    int4 vc[kBtViews];           // position of pixel (8, 8), its steps along x and y, and A
-    float2 a12[kBtViews];        // 1 + A, 1 - 2 A
+    int4 vc[kBtViews];           // position of pixel (8, 8), its steps along x and y, and A per position unit
+    float om[kBtViews];          // 1 - A
     float2 low[kBtViews];        // first staged ray (int bits), path length per step
     unsigned s_max;
     float s_tau_r;
 };
 
+// View (from v0) in slot i of a chunk of cnt views, cnt or more for a slot left
+// empty: a partial sum's kBtUnroll slots take views spread evenly over the
+// chunk, so that partial sums of a signed sinogram stay near their share of the
+// pixel's value.
+__device__ __forceinline__ int bt_view(int i, int cnt) {
+    const int parts = (cnt + kBtUnroll - 1) / kBtUnroll;
+    return i < parts * kBtUnroll ? (i & (kBtUnroll - 1)) * parts + i / kBtUnroll : kBtViews;
+}
+
 // Constants of views v0 .. v0 + cnt - 1 for the tile at (tx0, ty0).
 __device__ __forceinline__ void bt_view_setup(const ViewConst* __restrict__ vcs, int v0, int cnt, int tx0, int ty0,
                                               BtShared& sh) {
     for (int i = threadIdx.x; i < kBtViews; i += kBtWork) {
-        if (i >= cnt) {              // pads the last kBtUnroll views: no rays, all values 0
+        const int k = bt_view(i, cnt);
+        if (k >= cnt) {              // pads the partial sums: no rays, all values 0
             sh.vc[i] = make_int4(0, 0, 0, 0);
-            sh.a12[i] = make_float2(0.f, 0.f);
+            sh.om[i] = 0.f;
             sh.low[i] = make_float2(__int_as_float(INT_MIN / 2), 0.f);
             continue;
         }
-        const ViewConst& c = vcs[v0 + i];
+        const ViewConst& c = vcs[v0 + k];
         const long long qx = c.QX, qy = c.QY, h = kBtS / 2;
         const long long qc = c.Q0 + (tx0 + h) * qx + (ty0 + h) * qy;
         const long long ext = h * ((qx < 0 ? -qx : qx) + (qy < 0 ? -qy : qy));
         const long long lo = ((qc - ext) >> kQFrac) - 1;      // below every pixel's q by at least one bin
         constexpr int drop = kQFrac - kBtFrac;
         constexpr long long half = 1ll << (drop - 1);
-        // + half a unit of the 23 bits that become the float's mantissa
-        const int base = (int)((qc - (lo << kQFrac) + half) >> drop) + (1 << (kBtFrac - 24));
-        sh.vc[i] = make_int4(base, (int)((qx + half) >> drop), (int)((qy + half) >> drop),
-                             __float_as_int(fabsf(c.a_det)));
+        const int base = (int)((qc - (lo << kQFrac) + half) >> drop);
         const float A = fabsf(c.a_det);
-        sh.a12[i] = make_float2(1.f + A, 1.f - (A + A));
+        sh.vc[i] = make_int4(base, (int)((qx + half) >> drop), (int)((qy + half) >> drop),
+                             __float_as_int(A * (1.f / (float)(1 << kBtFrac))));      // exact: a power of two
+        sh.om[i] = 1.f - A;
         sh.low[i] = make_float2(__int_as_float((int)lo), c.w);
     }
 }
@@ -509,7 +525,7 @@ __device__ __forceinline__ bool bt_stage(const T* __restrict__ sino, int v0, int
             const float2 lw = sh.low[i];
             const int d = __float_as_int(lw.x) + lane;
             v[k] = 0.f;
-            if ((unsigned)d < (unsigned)nd) v[k] = ldf(sino + (size_t)(v0 + i) * nd + d) * lw.y;
+            if ((unsigned)d < (unsigned)nd) v[k] = ldf(sino + (size_t)(v0 + bt_view(i, cnt)) * nd + d) * lw.y;
         }
 #pragma unroll
         for (int k = 0; k < kBtBatch; ++k) {
@@ -540,30 +556,35 @@ __device__ __forceinline__ bool bt_sync_or(bool p) {
 // acc += the taps of a pixel at position q (both rays of the view).  SAFE:
 // a ray of weight 0 adds nothing even if its value is infinite or NaN.
 template <bool SAFE>
-__device__ __forceinline__ void bt_tap(const float2* __restrict__ seg, unsigned q, float A, float2 a12, float& acc) {
+__device__ __forceinline__ void bt_tap(const float2* __restrict__ seg, unsigned q, float A, float om, float& acc) {
     const float2 v = seg[q >> kBtFrac];
-    // 1 + fraction of q from its top 23 fraction bits
-    const float f = __uint_as_float(0x3F800000u | ((q >> (kBtFrac - 23)) & 0x7FFFFFu));
-    const float w0 = __saturatef(fmaf(-A, f, a12.x)), w1 = __saturatef(fmaf(A, f, a12.y));
+    const float f = __uint2float_rn(q & ((1u << kBtFrac) - 1u));      // the fraction, in position units
+    const float w0 = __saturatef(fmaf(-A, f, 1.f)), w1 = __saturatef(fmaf(A, f, om));
     if (!SAFE || w0 > 0.f) acc = fmaf(w0, v.x, acc);
     if (!SAFE || w1 > 0.f) acc = fmaf(w1, v.y, acc);
 }
 
 template <bool SAFE>
 __device__ __forceinline__ void bt_views(const BtShared& sh, int cnt, int lx, int ly, float& acc0, float& acc1) {
+    float g0 = 0.f, g1 = 0.f;
     for (int i0 = 0; i0 < cnt; i0 += kBtUnroll) {
         float t0 = 0.f, t1 = 0.f;
 #pragma unroll
         for (int k = 0; k < kBtUnroll; ++k) {
             const int4 c = sh.vc[i0 + k];
-            const float2 a12 = sh.a12[i0 + k];
+            const float om = sh.om[i0 + k];
             const float A = __int_as_float(c.w);
             const unsigned q = (unsigned)c.x + (unsigned)(lx * c.y) + (unsigned)(ly * c.z);
-            bt_tap<SAFE>(sh.seg[i0 + k], q, A, a12, t0);
-            bt_tap<SAFE>(sh.seg[i0 + k], q + 8u * (unsigned)c.z, A, a12, t1);
+            bt_tap<SAFE>(sh.seg[i0 + k], q, A, om, t0);
+            bt_tap<SAFE>(sh.seg[i0 + k], q + 8u * (unsigned)c.z, A, om, t1);
         }
-        acc0 += t0;
-        acc1 += t1;
+        g0 += t0;
+        g1 += t1;
+        if ((i0 & (kBtGroup - kBtUnroll)) == kBtGroup - kBtUnroll || i0 + kBtUnroll >= cnt) {
+            acc0 += g0;
+            acc1 += g1;
+            g0 = g1 = 0.f;
+        }
     }
 }
 
