@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(512) k_batch_vinv_rows(const BatchSlice* __res
                                                          const uint16_t* __restrict__ map) {
     extern __shared__ float2 smem[];
     const BatchSlice& B = sl[map[blockIdx.x]];
-    img_rows_fwd_block(B.x, B.n, B.m2, 2 * ((int)blockIdx.x - B.off[kPhRow]), B.tw2, B.fft2d, smem);
+    img_rows_fwd_block(B.x, B.n, B.m2, (int)blockIdx.x - B.off[kPhRow], B.tw2, B.fft2d, smem);
 }
 
 __global__ void __launch_bounds__(512) k_batch_vinv_cols(const BatchSlice* __restrict__ sl,
@@ -191,15 +191,11 @@ __global__ void __launch_bounds__(512) k_batch_vinv_rows_inv(const BatchSlice* _
                                                              const uint16_t* __restrict__ map) {
     extern __shared__ float2 smem[];
     const BatchSlice& B = sl[map[blockIdx.x]];
-    const int y0 = 2 * ((int)blockIdx.x - B.off[kPhRow]), n = B.n;
-    const float2* r = img_rows_inv_block(B.fft2d, n, B.m2, y0, B.tw2, smem);
+    const int y = (int)blockIdx.x - B.off[kPhRow], n = B.n;
+    const float2* r = img_rows_inv_block(B.fft2d, B.m2, y, B.tw2, smem);
     const float sc = 1.0f / ((float)B.m2 * (float)B.m2);
-    float* __restrict__ out = B.mu_out + (size_t)y0 * n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float2 v = r[fpad(i)];
-        out[i] = v.x * sc;
-        if (y0 + 1 < n) out[n + i] = v.y * sc;
-    }
+    float* __restrict__ out = B.mu_out + (size_t)y * n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = r[fpad(i)].x * sc;
 }
 
 }  // namespace dgct
@@ -391,7 +387,7 @@ int dgamp_ct_batch_create(int32_t n, const dgamp_ct_plan_t* plans, int32_t group
         const long long begin_elems = std::max<long long>(std::max<long long>(pl->M, pl->N), (long long)pl->n * pl->ldp);
         const int cnt[kPhases] = {batch_grid_project(pl->nv, pl->nd), pl->nv, batch_grid_backproject(pl->n),
                                   batch_grid_probe(pl->N), batch_grid_tv(pl->n, 0), batch_grid_tv(pl->n, 1),
-                                  (pl->n + 1) / 2, img_col_blocks(pl->m2, vinv_nc), (int)((begin_elems + 255) / 256)};
+                                  pl->n, pl->m2 / vinv_nc, (int)((begin_elems + 255) / 256)};
         const int gk = group_of[i];
         for (int ph = 0; ph < kPhases; ++ph) {
             auto& mp = (ph == kPhRow || ph == kPhCol || ph == kPhBegin) ? maps[ph] : gmaps[gk][ph];

@@ -274,15 +274,14 @@ int toeplitz_set_smem_limit(int nd) {
 }
 
 // ------------------------------------------------------- V^-1 / V image --
-// Image blockIdx.y of a batch (img and out [nimg][n][n], C [nimg][n][img_stride(m)]);
+// Image blockIdx.y of a batch (img and out [nimg][n][n], C [nimg][n][m]);
 // a single image is the batch of one.  The passes are in fft_device.cuh.
 __global__ void __launch_bounds__(512)
 k_img_rows_fwd(const float* __restrict__ img, int n, int m, const float2* __restrict__ tw,
                float2* __restrict__ C) {
     extern __shared__ float2 smem[];
     pdl_wait();
-    img_rows_fwd_block(img + (size_t)blockIdx.y * n * n, n, m, 2 * blockIdx.x, tw,
-                       C + (size_t)blockIdx.y * n * img_stride(m), smem);
+    img_rows_fwd_block(img + (size_t)blockIdx.y * n * n, n, m, blockIdx.x, tw, C + (size_t)blockIdx.y * n * m, smem);
 }
 
 __global__ void __launch_bounds__(512)
@@ -290,28 +289,24 @@ k_img_cols(float2* __restrict__ C, int n, int m, const float2* __restrict__ tw, 
            int inverse_gain) {
     extern __shared__ float2 smem[];
     pdl_wait();
-    img_cols_block(C + (size_t)blockIdx.y * n * img_stride(m), n, m, blockIdx.x, tw, f0, inverse_gain, smem);
+    img_cols_block(C + (size_t)blockIdx.y * n * m, n, m, blockIdx.x, tw, f0, inverse_gain, smem);
 }
 
-// pass 3: inverse row FFTs, the first n columns, scaled by 1/m^2.
+// pass 3: inverse row FFTs, real part of the first n columns, scaled by 1/m^2.
 __global__ void __launch_bounds__(512)
 k_img_rows_inv(const float2* __restrict__ C, int n, int m, const float2* __restrict__ tw,
                float* __restrict__ out) {
     extern __shared__ float2 smem[];
-    const int y0 = 2 * blockIdx.x;
+    const int y = blockIdx.x;
     pdl_wait();
-    const float2* r = img_rows_inv_block(C + (size_t)blockIdx.y * n * img_stride(m), n, m, y0, tw, smem);
-    out += (size_t)blockIdx.y * n * n + (size_t)y0 * n;
+    const float2* r = img_rows_inv_block(C + (size_t)blockIdx.y * n * m, m, y, tw, smem);
+    out += (size_t)blockIdx.y * n * n + (size_t)y * n;
     const float sc = 1.0f / ((float)m * (float)m);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float2 v = r[fpad(i)];
-        out[i] = v.x * sc;
-        if (y0 + 1 < n) out[n + i] = v.y * sc;
-    }
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = r[fpad(i)].x * sc;
 }
 
 // pass 3 of V^-1 inside a fan-beam solve (Algorithm 1, Step 3 with
-// Phi~^T = V^-1 A^T): r = x + tau_r (.) / m^2 with tau_r from the device
+// Phi~^T = V^-1 A^T): r = x + tau_r Re(.) / m^2 with tau_r from the device
 // scalars (the output step formed it), max |r| into S->rmax_bits (the output
 // step reset it), and the consumed divergence flag cleared, as the
 // parallel-beam back-projection does.
@@ -320,22 +315,19 @@ k_img_rows_inv_update(const float2* __restrict__ C, int n, int m, const float2* 
                       const float* __restrict__ x, DevScalars* __restrict__ S, float* __restrict__ out) {
     extern __shared__ float2 smem[];
     __shared__ unsigned s_max;
-    const int y0 = 2 * blockIdx.x;
+    const int y = blockIdx.x;
     pdl_wait();
     if (threadIdx.x == 0) {
         s_max = 0u;
-        if (y0 == 0) S->div_pending = 0u;
+        if (y == 0) S->div_pending = 0u;
     }
-    const float2* r = img_rows_inv_block(C, n, m, y0, tw, smem);
+    const float2* r = img_rows_inv_block(C, m, y, tw, smem);
     const float sc = (float)S->tau_r / ((float)m * (float)m);
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float2 v = r[fpad(i)];
-        for (int h = 0; h < 2 && y0 + h < n; ++h) {
-            const size_t o = (size_t)(y0 + h) * n + i;
-            const float rv = fmaf(sc, h ? v.y : v.x, x[o]);
-            out[o] = rv;
-            atomicMax(&s_max, __float_as_uint(fabsf(rv)));   // |r| >= 0: bit order is value order
-        }
+        const size_t o = (size_t)y * n + i;
+        const float rv = fmaf(sc, r[fpad(i)].x, x[o]);
+        out[o] = rv;
+        atomicMax(&s_max, __float_as_uint(fabsf(rv)));   // |r| >= 0: bit order is value order
     }
     __syncthreads();
     if (threadIdx.x == 0) atomicMax(&S->rmax_bits, s_max);
@@ -347,9 +339,9 @@ static int launch_img_forward(const dgamp_ct_plan_s* pl, const float* in, float2
     const int n = pl->n, m = pl->m2, thr = fft_threads(m), nc = img_cols_per_block(m);
     const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
     const float f0 = 1.0f / (2.0f * (float)pl->P);
-    DGCT_CUDA(launch_pdl(k_img_rows_fwd, dim3((n + 1) / 2, nimg), dim3(thr), sm, st, in, n, m, pl->ws.tw2, C));
+    DGCT_CUDA(launch_pdl(k_img_rows_fwd, dim3(n, nimg), dim3(thr), sm, st, in, n, m, pl->ws.tw2, C));
     // V^-1 applies sqrt(max(rho, f0)); V applies its reciprocal
-    DGCT_CUDA(launch_pdl(k_img_cols, dim3(img_col_blocks(m, nc), nimg), dim3(thr, nc), nc * sm, st, C, n, m, pl->ws.tw2,
+    DGCT_CUDA(launch_pdl(k_img_cols, dim3(m / nc, nimg), dim3(thr, nc), nc * sm, st, C, n, m, pl->ws.tw2,
                          f0, inverse_gain));
     return DGAMP_CT_OK;
 }
@@ -359,7 +351,7 @@ int launch_precond_image_update(const dgamp_ct_plan_s* pl, const float* in, cons
     const int n = pl->n, m = pl->m2;
     const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
     DGCT_TRY(launch_img_forward(pl, in, pl->ws.fft2d, 1, 0, st));
-    DGCT_CUDA(launch_pdl(k_img_rows_inv_update, dim3((n + 1) / 2), dim3(fft_threads(m)), sm, st, pl->ws.fft2d, n, m,
+    DGCT_CUDA(launch_pdl(k_img_rows_inv_update, dim3(n), dim3(fft_threads(m)), sm, st, pl->ws.fft2d, n, m,
                          pl->ws.tw2, x, pl->ws.S, out));
     return DGAMP_CT_OK;
 }
@@ -370,15 +362,15 @@ int launch_precond_image(const dgamp_ct_plan_s* pl, const float* in, float* out,
 }
 
 // nimg images at once ([nimg][n][n] in and out) through the scratch C
-// ([nimg][n][m2] complex at least, the caller's); the same kernels and
-// arithmetic per image as launch_precond_image
+// ([nimg][n][m2] complex, the caller's); the same kernels and arithmetic per
+// image as launch_precond_image
 int launch_precond_images(const dgamp_ct_plan_s* pl, const float* in, float* out, float2* C, int nimg, int inverse,
                           cudaStream_t st) {
     if (nimg < 1) return DGAMP_CT_ERR_INVALID_ARG;
     const int n = pl->n, m = pl->m2;
     const size_t sm = (size_t)2 * fft_buf_len(m) * sizeof(float2);
     DGCT_TRY(launch_img_forward(pl, in, C, nimg, inverse ? 0 : 1, st));
-    DGCT_CUDA(launch_pdl(k_img_rows_inv, dim3((n + 1) / 2, nimg), dim3(fft_threads(m)), sm, st, C, n, m, pl->ws.tw2, out));
+    DGCT_CUDA(launch_pdl(k_img_rows_inv, dim3(n, nimg), dim3(fft_threads(m)), sm, st, C, n, m, pl->ws.tw2, out));
     return DGAMP_CT_OK;
 }
 

@@ -136,55 +136,47 @@ __device__ __forceinline__ float2* fft_stockham(float2* a, float2* b, int P, con
 
 // ------------------------------------------------ V^-1 / V of an image --
 // The 2-D filter of an n x n real image on its m x m zero-padded grid, in three
-// passes over the spectrum C [n][img_stride(m)] (frequencies 0 .. m/2 of each
-// row: the rest mirrors them), shared by the single and the batched kernels.
-// Rows run two at a time as one complex line (real + i imaginary).  Against
-// one row per transform and all m columns, every pass does half the transforms
-// and moves half the bytes; a block takes NC neighbouring columns, so that the
-// row-major spectrum is read in whole sectors.  Fan-beam A + A^T at
-// 512^2/102/736, which filters twice: 224 -> 210 us.
-__host__ __device__ __forceinline__ int img_stride(int m) { return m >= 8 ? m / 2 + 4 : m; }
+// passes over the spectrum C [n][m], shared by the single and the batched
+// kernels: rows, columns with the radial gain between their forward and inverse
+// transforms, rows back.  A block takes NC neighbouring columns, so that the
+// row-major spectrum is read in whole sectors.  The rows' conjugate symmetry is
+// not used: two rows as one complex line and half the columns halve the work,
+// but the error of V^-1 x against 64 bits grows by a quarter (2.0e-7 -> 2.5e-7
+// over 64^2 .. 1024^2), since the discarded imaginary parts and the mirrored
+// frequencies then no longer take their share of the rounding.
 __host__ __device__ __forceinline__ int img_cols_per_block(int m) { return m <= 1024 ? 4 : (m <= 2048 ? 2 : 1); }
-__host__ __device__ __forceinline__ int img_col_blocks(int m, int nc) { return (m / 2 + nc) / nc; }
 
-// rows y0, y0 + 1 of img -> C
-__device__ __forceinline__ void img_rows_fwd_block(const float* __restrict__ img, int n, int m, int y0,
+// row y of img -> C
+__device__ __forceinline__ void img_rows_fwd_block(const float* __restrict__ img, int n, int m, int y,
                                                    const float2* __restrict__ tw, float2* __restrict__ C,
                                                    float2* smem) {
     float2* a = smem;
     float2* b = smem + fft_buf_len(m);
-    const bool two = y0 + 1 < n;
-    const float* __restrict__ row = img + (size_t)y0 * n;
     for (int i = threadIdx.x; i < m; i += blockDim.x)
-        a[fpad(i)] = i < n ? make_float2(row[i], two ? row[n + i] : 0.f) : make_float2(0.f, 0.f);
+        a[fpad(i)] = make_float2(i < n ? img[(size_t)y * n + i] : 0.f, 0.f);
     __syncthreads();
     const float2* r = fft_stockham(a, b, m, tw, -1.f);
-    float2* __restrict__ c0 = C + (size_t)y0 * img_stride(m);
-    for (int k = threadIdx.x; k <= m / 2; k += blockDim.x) {
-        const float2 z = r[fpad(k)], y = r[fpad((m - k) & (m - 1))];
-        c0[k] = make_float2(0.5f * (z.x + y.x), 0.5f * (z.y - y.y));
-        if (two) c0[img_stride(m) + k] = make_float2(0.5f * (z.y + y.y), 0.5f * (y.x - z.x));
-    }
+    for (int i = threadIdx.x; i < m; i += blockDim.x) C[(size_t)y * m + i] = r[fpad(i)];
 }
 
-// columns NC bx + threadIdx.y (blockDim.y = NC): forward transform over the
-// rows (rows >= n are zero), radial gain sqrt(max(rho, f0)) or its reciprocal,
-// inverse transform; rows < n are stored back.
+// columns NC bx + threadIdx.y (blockDim.y = NC, which divides m): forward
+// transform over the rows (rows >= n are zero), radial gain sqrt(max(rho, f0))
+// or its reciprocal, inverse transform; rows < n are stored back.
 __device__ __forceinline__ void img_cols_block(float2* __restrict__ C, int n, int m, int bx,
                                                const float2* __restrict__ tw, float f0, int inverse_gain,
                                                float2* smem) {
-    const int NC = blockDim.y, kx0 = bx * NC, ms = img_stride(m), BL = fft_buf_len(m);
+    const int NC = blockDim.y, kx0 = bx * NC, BL = fft_buf_len(m);
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * NC, sh = __ffs(NC) - 1;   // NC = 1, 2, 4
     for (int j = tid; j < m * NC; j += nt) {       // NC columns of a row are neighbours in memory
         const int i = j >> sh, c = j & (NC - 1);
-        smem[2 * c * BL + fpad(i)] =
-            i < n && kx0 + c <= m / 2 ? C[(size_t)i * ms + kx0 + c] : make_float2(0.f, 0.f);
+        smem[2 * c * BL + fpad(i)] = i < n ? C[(size_t)i * m + kx0 + c] : make_float2(0.f, 0.f);
     }
     __syncthreads();
     float2* a = smem + 2 * threadIdx.y * BL;
     float2* r = fft_stockham(a, a + BL, m, tw, -1.f);
     float2* o = (r == a) ? a + BL : a;
-    const float fx = (float)(kx0 + threadIdx.y) / (float)m;
+    const int kx = kx0 + threadIdx.y;
+    const float fx = (float)(kx <= m / 2 ? kx : kx - m) / (float)m;
     for (int ky = threadIdx.x; ky < m; ky += blockDim.x) {
         const float fy = (float)(ky <= m / 2 ? ky : ky - m) / (float)m;
         const float rho = sqrtf(fx * fx + fy * fy);
@@ -198,23 +190,17 @@ __device__ __forceinline__ void img_cols_block(float2* __restrict__ C, int n, in
     const int at = (int)(r - a);                   // the same buffer of every column
     for (int j = tid; j < n * NC; j += nt) {
         const int i = j >> sh, c = j & (NC - 1);
-        if (kx0 + c <= m / 2) C[(size_t)i * ms + kx0 + c] = smem[2 * c * BL + at + fpad(i)];
+        C[(size_t)i * m + kx0 + c] = smem[2 * c * BL + at + fpad(i)];
     }
 }
 
-// inverse transforms of rows y0, y0 + 1: their first n values (times m^2) are
-// the real and imaginary parts of the returned buffer
-__device__ __forceinline__ const float2* img_rows_inv_block(const float2* __restrict__ C, int n, int m, int y0,
+// inverse transform of row y: its first n values (times m^2) are the real parts
+// of the returned buffer
+__device__ __forceinline__ const float2* img_rows_inv_block(const float2* __restrict__ C, int m, int y,
                                                             const float2* __restrict__ tw, float2* smem) {
     float2* a = smem;
     float2* b = smem + fft_buf_len(m);
-    const bool two = y0 + 1 < n;
-    const float2* __restrict__ c0 = C + (size_t)y0 * img_stride(m);
-    for (int k = threadIdx.x; k <= m / 2; k += blockDim.x) {
-        const float2 f = c0[k], g = two ? c0[img_stride(m) + k] : make_float2(0.f, 0.f);
-        a[fpad(k)] = make_float2(f.x - g.y, f.y + g.x);
-        if (k > 0 && k < m / 2) a[fpad(m - k)] = make_float2(f.x + g.y, g.x - f.y);
-    }
+    for (int i = threadIdx.x; i < m; i += blockDim.x) a[fpad(i)] = C[(size_t)y * m + i];
     __syncthreads();
     return fft_stockham(a, b, m, tw, 1.f);
 }
