@@ -217,9 +217,11 @@ int dgamp_ct_plan_info(dgamp_ct_plan_t plan, double* frob_sq, int32_t* fft_len);
 typedef struct {
     int32_t filter_mode;  /* 0 = H by FFT, 1 = H as a Toeplitz product with the same
                              kernel h = IFFT_P(g) (no wrap-around since P >= 2 n_det).
-                             Reported for the single-step calls; inside a solve's
-                             three-kernel form H runs by FFT, with output_moments = 1 in the
-                             faster form, unless this is set */
+                             The form of the single-step calls and of a solve's three
+                             kernels, with one exception: a Laplace solve
+                             (output_moments = 0) told to run three kernels takes the FFT,
+                             as the fused form 1 does, until set_tuning has changed this
+                             field (setting the value that get reports changes nothing) */
     int32_t tv_kb;        /* Chambolle steps per blocked TV launch, 1..10 */
     int32_t tv_rows;      /* rows of the image region one TV block holds: 32, 64 or 128
                              (the region is 64 columns wide) */
@@ -228,9 +230,9 @@ typedef struct {
                              P <= 8192); 2 = a cluster of 8 blocks per view, each a slice
                              of the bins, H as its Toeplitz product and s shared through
                              distributed shared memory (needs n_det <= 1792); 0 = three
-                             kernels, H as filter_mode says.  The plan times the forms
-                             the geometry allows and keeps the faster; filter_mode alone
-                             governs the single-step entry points */
+                             kernels, H as described at filter_mode.  The plan times the
+                             forms the geometry allows and keeps the faster; filter_mode
+                             alone governs the single-step entry points */
     int32_t bp_mode;      /* A^T: 0 = pixel-driven gather (each pixel finds the <= 2 rays
                              of a view that tap it and takes the projector's own weights),
                              1 = 16 x 16 image tiles that stage the rays of 64 views in

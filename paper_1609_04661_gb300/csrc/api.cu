@@ -22,7 +22,7 @@ int cuda_fail(cudaError_t e) {
 
 static void free_ws(Workspace& w) {
     void* ptrs[] = {w.XR, w.XC, w.x, w.r, w.b, w.p, w.zraw, w.z, w.s, w.hs, w.y, w.fft2d, w.partial,
-                    w.partial_div, w.S, w.log, w.vc, w.gain, w.tw, w.tw2, w.twh, w.scratch_d, w.hx, w.zraw2,
+                    w.partial_div, w.S, w.log, w.vc, w.gain, w.tw, w.tw2, w.scratch_d, w.hx, w.zraw2,
                     w.fan_rays, w.fan_views, w.fan_gw, w.pj_order, w.pj_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -137,7 +137,6 @@ static int plan_alloc(dgamp_ct_plan_s* pl, const std::vector<double>& ang) {
     DGCT_TRY(dalloc(&w.gain, (size_t)pl->P));
     DGCT_TRY(dalloc(&w.tw, (size_t)fft_twiddle_count(pl->P) + 1));
     DGCT_TRY(dalloc(&w.tw2, (size_t)fft_twiddle_count(pl->m2) + 1));
-    DGCT_TRY(dalloc(&w.twh, (size_t)fft_twiddle_count(pl->P / 2) + 1));
     DGCT_TRY(dalloc(&w.hx, (size_t)2 * pl->nd));
     DGCT_TRY(dalloc(&w.zraw2, M));
     DGCT_TRY(dalloc(&w.scratch_d, (size_t)(pl->nd + 1) + 2 * pl->nd + pl->nv + (size_t)pl->nv * pl->nd));
@@ -203,7 +202,6 @@ static int plan_alloc(dgamp_ct_plan_s* pl, const std::vector<double>& ang) {
     };
     DGCT_TRY(twiddles(P, w.tw));
     DGCT_TRY(twiddles(pl->m2, w.tw2));
-    DGCT_TRY(twiddles(P / 2, w.twh));
 
     // ||Phi~||_F^2 on the device in FP64
     double* ang_dev = w.scratch_d + (pl->nd + 1) + 2 * pl->nd;
@@ -599,7 +597,10 @@ int dgamp_ct_set_tuning(dgamp_ct_plan_t pl, const dgamp_ct_tuning* t) {
     if (t->sino_fused == 1 && !sino_step_eligible(pl)) return DGAMP_CT_ERR_UNSUPPORTED_GEOMETRY;
     if (t->sino_fused == 2 && !sino_toeplitz_eligible(pl)) return DGAMP_CT_ERR_UNSUPPORTED_GEOMETRY;
     if (pl->fan && t->bp_mode == 1 && pl->fan_stride <= 0) return DGAMP_CT_ERR_UNSUPPORTED_GEOMETRY;
-    if (t->filter_mode >= 0) pl->filter_mode = pl->filter_set = t->filter_mode;
+    if (t->filter_mode >= 0 && t->filter_mode != pl->filter_mode) {   // writing back what get reported sets nothing
+        pl->filter_mode = t->filter_mode;
+        pl->filter_set = 1;
+    }
     if (t->tv_kb > 0) pl->tv_kb = t->tv_kb;
     if (t->tv_rows > 0) pl->tv_rows = t->tv_rows;
     if (t->sino_fused >= 0) pl->sino_fused = t->sino_fused;

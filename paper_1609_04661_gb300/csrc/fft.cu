@@ -1,8 +1,9 @@
 // Shared-memory FFTs for the Radon preconditioner (Section 2.4, Eq. Aprecon).
 //
-//  * H on sinograms: one block per view, the real line of length P as a complex
-//    one of length P/2 (even bins + i odd bins), split into the spectra of the
-//    even and odd bins for the gain and put together again.
+//  * H on sinograms: one block filters two views at once, packed as the real
+//    and imaginary parts of one complex line.  Because the gain g is real and
+//    even, filtering a + i b gives H a + i H b, so one forward and one inverse
+//    complex FFT of length P serve two views.
 //  * V^-1 / V on images: a 2-D zero-padded FFT done as row FFTs, column FFTs
 //    with the radial gain applied between the forward and inverse column
 //    transforms, and inverse row FFTs.  It runs once per solve.
@@ -19,68 +20,14 @@ namespace dgct {
 static int fft_threads(int P) { return P / 8 < 32 ? 32 : (P / 8 > 512 ? 512 : P / 8); }
 
 // ------------------------------------------------------------ H on views --
-// One view per block.  With z[j] = x[2j] + i x[2j + 1] and Z its DFT of length
-// L = P / 2, the even and odd bins' DFTs are E = (Z[k] + conj Z[L-k]) / 2 and
-// O = (Z[k] - conj Z[L-k]) / 2i, and x's own are E +- w^k O at k and k + L,
-// w = exp(-2 pi i / P).  With these times the gains g[k] and g[k + L] = g[L-k] as
-// A and C, E' = (A + C) / 2 and O' = w^-k (A - C) / 2, and Z' = E' + i O' (at L-k:
-// conj E' + i conj O') transforms back to the filtered bins.  (Gathering E and O
-// by (g[k] +- g[L-k]) instead saves an addition each, but lets the high
-// frequencies' rounding into the low ones, which A^T then amplifies.)  The block's chain of stages and barriers bounds the kernel,
-// not its arithmetic: a pair of views per block as one complex line of length P
-// left 45 blocks with twice the butterflies per stage at 90 views, P = 4096.
-// Two filters and an output step at 90 x 1449: 55.5 -> 50.2 us.
-__global__ void __launch_bounds__(512)
-k_filter_line(const float* in, float* out, int nd, int P, const float* __restrict__ gain, const float2* __restrict__ tw) {
-    extern __shared__ float2 smem[];
-    const int L = P >> 1;
-    float2* a = smem;
-    float2* b = smem + fft_buf_len(L);
-    const float* row = in + (size_t)blockIdx.x * nd;
-    pdl_wait();
-    for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        float2 v = make_float2(0.f, 0.f);
-        if (2 * i < nd) v.x = row[2 * i];
-        if (2 * i + 1 < nd) v.y = row[2 * i + 1];
-        a[fpad(i)] = v;
-    }
-    __syncthreads();
-    float2* r = fft_stockham(a, b, L, tw, -1.f);
-    float2* o = (r == a) ? b : a;
-    const float sc = 0.25f / (float)L;      // the two halvings above, and 1 / L of the inverse
-    for (int k = threadIdx.x; k <= L / 2; k += blockDim.x) {
-        const int kk = (L - k) & (L - 1);
-        const float2 z = r[fpad(k)], y = r[fpad(kk)];
-        const float ga = __ldg(gain + k) * sc, gb = __ldg(gain + L - k) * sc;
-        float sn, cs;
-        sincospif((float)k / (float)L, &sn, &cs);                    // w^k = cs - i sn
-        const float2 E = make_float2(z.x + y.x, z.y - y.y), O = make_float2(z.y + y.y, y.x - z.x);   // twice E, O
-        const float2 wO = make_float2(fmaf(cs, O.x, sn * O.y), fmaf(cs, O.y, -sn * O.x));
-        const float2 A = make_float2(ga * (E.x + wO.x), ga * (E.y + wO.y));
-        const float2 C = make_float2(gb * (E.x - wO.x), gb * (E.y - wO.y));
-        const float2 e = cadd(A, C), d = csub(A, C);
-        const float2 q = make_float2(fmaf(cs, d.x, -sn * d.y), fmaf(cs, d.y, sn * d.x));             // w^-k (A - C)
-        r[fpad(k)] = make_float2(e.x - q.y, e.y + q.x);
-        if (kk != k) r[fpad(kk)] = make_float2(e.x + q.y, q.x - e.y);
-    }
-    __syncthreads();
-    r = fft_stockham(r, o, L, tw, 1.f);
-    float* w = out + (size_t)blockIdx.x * nd;
-    for (int i = threadIdx.x; i < nd; i += blockDim.x) {
-        const float2 v = r[fpad(i >> 1)];
-        w[i] = (i & 1) ? v.y : v.x;
-    }
-}
-
 // Two views per block as one complex line of length P, which the real and even
-// gain filters both: the arithmetic of the fused sinogram kernel's FFT form.  A
-// solve in the three-kernel form takes this one, so that the two forms' scalars
-// stay together over the iterations (on the smallest geometries the half-length
-// line's rounding grows past 1e-4 in five); single-step calls take the faster
-// line per view above.
+// gain filters both: the arithmetic of the fused sinogram kernel's FFT form.
+// (One view as a complex line of half the length was no faster, 52.6 against
+// 51.7 us for two filters and an output step at 90 x 1449 where runs differ by
+// 15%, and 4-5% further from 64 bits.)
 template <typename T>
 __global__ void __launch_bounds__(512)
-k_filter_pairs(const T* in, T* out, int nv, int nd, int P,
+k_filter_views(const T* in, T* out, int nv, int nd, int P,
                const float* __restrict__ gain, const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
     float2* a = smem;
@@ -89,6 +36,7 @@ k_filter_pairs(const T* in, T* out, int nv, int nd, int P,
     const bool hasb = vb < nv;
     const T* ra = in + (size_t)va * nd;
     const T* rb = in + (size_t)vb * nd;
+    pdl_wait();
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         float2 v = make_float2(0.f, 0.f);
         if (i < nd) {
@@ -184,83 +132,73 @@ static size_t toeplitz_smem(int nd) {
     return ((size_t)nd + 2 * nd - 1 + kTzWarps * kTzOut) * sizeof(float);
 }
 
+// H's form for launch_filter.  The single steps, and a solve with exact moments,
+// take the plan's timed choice.  A Laplace solve runs the three kernels only if
+// told to (sino_fused = 0), beside the fused FFT form, and takes the FFT as well
+// unless the tuning has set a form: then the two forms agree bit for bit, where
+// the Toeplitz product's order of summation parts them by up to 1.5e-4 in tau_r
+// over five iterations of a 16 x 16 image (3 views of 24 bins).
+static bool filter_by_toeplitz(const dgamp_ct_plan_s* pl, int solve) {
+    if (solve && !pl->opt.output_moments && !pl->filter_set) return false;
+    return pl->filter_mode == 1;
+}
+
 // bf = 1: in and out hold BF16 (a solve with storage = 1); sums in FP32 either way
 int launch_filter(const dgamp_ct_plan_s* pl, const float* in, float* out, cudaStream_t st, int bf, int solve) {
-    // A solve's three-kernel form: with the Laplace step it stands beside the fused FFT form and takes its
-    // arithmetic (k_filter_pairs) unless the tuning sets one; with exact moments it is the only form there is
-    // and takes the faster
-    const int in_solve = pl->filter_set >= 0 ? pl->filter_set : (pl->opt.output_moments ? pl->filter_solve : 0);
-    if ((solve ? in_solve : pl->filter_mode) == 1) {
+    if (filter_by_toeplitz(pl, solve)) {
         // the block reads its whole input row first, so in == out needs a copy
         const float* src = in;
         if (in == out) {
             DGCT_CUDA(cudaMemcpyAsync(pl->ws.zraw2, in, (size_t)pl->M * (bf ? 2 : 4), cudaMemcpyDeviceToDevice, st));
             src = pl->ws.zraw2;
         }
-        dim3 grd((pl->nd + kTzOut - 1) / kTzOut, pl->nv);
+        const dim3 grd((pl->nd + kTzOut - 1) / kTzOut, pl->nv), blk(32 * kTzWarps);
         const size_t sm = toeplitz_smem(pl->nd);
-        if (solve) {
-            if (bf)
-                k_filter_toeplitz<bf16s><<<grd, 32 * kTzWarps, sm, st>>>((const bf16s*)src, (bf16s*)out, pl->nd, pl->ws.hx);
-            else
-                k_filter_toeplitz<float><<<grd, 32 * kTzWarps, sm, st>>>(src, out, pl->nd, pl->ws.hx);
-            DGCT_LAUNCH_CHECK();
-        } else {
-            DGCT_CUDA(launch_pdl(k_filter_toeplitz<float>, grd, dim3(32 * kTzWarps), sm, st, src, out, pl->nd, pl->ws.hx));
-        }
-        return DGAMP_CT_OK;
-    }
-    if (solve) {
-        const size_t sm = (size_t)2 * fft_buf_len(pl->P) * sizeof(float2);
-        const dim3 grd((pl->nv + 1) / 2), blk(fft_threads(pl->P));
         if (bf)
-            k_filter_pairs<bf16s><<<grd, blk, sm, st>>>((const bf16s*)in, (bf16s*)out, pl->nv, pl->nd, pl->P, pl->ws.gain,
-                                                        pl->ws.tw);
+            DGCT_CUDA(launch_pdl(k_filter_toeplitz<bf16s>, grd, blk, sm, st, (const bf16s*)src, (bf16s*)out, pl->nd,
+                                 pl->ws.hx));
         else
-            k_filter_pairs<float><<<grd, blk, sm, st>>>(in, out, pl->nv, pl->nd, pl->P, pl->ws.gain, pl->ws.tw);
-        DGCT_LAUNCH_CHECK();
+            DGCT_CUDA(launch_pdl(k_filter_toeplitz<float>, grd, blk, sm, st, src, out, pl->nd, pl->ws.hx));
         return DGAMP_CT_OK;
     }
-    const int P = pl->P, L = P / 2;
-    const size_t sm = (size_t)2 * fft_buf_len(L) * sizeof(float2);
-    const int thr = fft_threads(L);
-    DGCT_CUDA(launch_pdl(k_filter_line, dim3(pl->nv), dim3(thr), sm, st, in, out, pl->nd, P, pl->ws.gain, pl->ws.twh));
+    const int P = pl->P;
+    const size_t sm = (size_t)2 * fft_buf_len(P) * sizeof(float2);
+    const dim3 grd((pl->nv + 1) / 2), blk(fft_threads(P));
+    if (bf)
+        DGCT_CUDA(launch_pdl(k_filter_views<bf16s>, grd, blk, sm, st, (const bf16s*)in, (bf16s*)out, pl->nv, pl->nd, P,
+                             pl->ws.gain, pl->ws.tw));
+    else
+        DGCT_CUDA(launch_pdl(k_filter_views<float>, grd, blk, sm, st, in, out, pl->nv, pl->nd, P, pl->ws.gain,
+                             pl->ws.tw));
     return DGAMP_CT_OK;
 }
 
-// Plan-time choice between the FFT and the Toeplitz form of H (same operator),
-// for the single-step calls and for a solve's three-kernel form: time both on
-// the plan's geometry and keep the faster.
+// Plan-time choice between the FFT and the Toeplitz form of H (same operator):
+// time both on the plan's geometry and keep the faster.
 int filter_autotune(dgamp_ct_plan_s* pl) {
     DGCT_CUDA(cudaMemset(pl->ws.zraw, 0, (size_t)pl->M * sizeof(float)));
     cudaEvent_t e0, e1;
     DGCT_CUDA(cudaEventCreate(&e0));
     DGCT_CUDA(cudaEventCreate(&e1));
-    int rc = DGAMP_CT_OK;
-    for (int solve = 0; solve < 2 && rc == DGAMP_CT_OK; ++solve) {
-        int& choice = solve ? pl->filter_solve : pl->filter_mode;
-        float best = 1e30f;
-        int best_mode = 0;
-        for (int mode = 0; mode < 2 && rc == DGAMP_CT_OK; ++mode) {
-            choice = mode;
-            pl->filter_set = solve ? mode : -1;
-            for (int rep = 0; rep < 6 && rc == DGAMP_CT_OK; ++rep) {
-                if (rep == 1) cudaEventRecord(e0, 0);
-                rc = launch_filter(pl, pl->ws.zraw, pl->ws.z, 0, 0, solve);
-            }
-            cudaEventRecord(e1, 0);
-            const cudaError_t e = cudaEventSynchronize(e1);
-            if (rc == DGAMP_CT_OK && e != cudaSuccess) rc = cuda_fail(e);
-            float ms = 0.f;
-            if (rc == DGAMP_CT_OK) cudaEventElapsedTime(&ms, e0, e1);
-            if (rc == DGAMP_CT_OK && ms < best) {
-                best = ms;
-                best_mode = mode;
-            }
+    float best = 1e30f;
+    int best_mode = 0, rc = DGAMP_CT_OK;
+    for (int mode = 0; mode < 2 && rc == DGAMP_CT_OK; ++mode) {
+        pl->filter_mode = mode;
+        for (int rep = 0; rep < 6 && rc == DGAMP_CT_OK; ++rep) {
+            if (rep == 1) cudaEventRecord(e0, 0);
+            rc = launch_filter(pl, pl->ws.zraw, pl->ws.z, 0);
         }
-        choice = best_mode;
+        cudaEventRecord(e1, 0);
+        const cudaError_t e = cudaEventSynchronize(e1);
+        if (rc == DGAMP_CT_OK && e != cudaSuccess) rc = cuda_fail(e);
+        float ms = 0.f;
+        if (rc == DGAMP_CT_OK) cudaEventElapsedTime(&ms, e0, e1);
+        if (rc == DGAMP_CT_OK && ms < best) {
+            best = ms;
+            best_mode = mode;
+        }
     }
-    pl->filter_set = -1;
+    pl->filter_mode = best_mode;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     return rc;
@@ -375,9 +313,8 @@ int launch_precond_images(const dgamp_ct_plan_s* pl, const float* in, float* out
 }
 
 int fft_set_smem_limits(int bytes) {
-    DGCT_TRY(raise_smem_limit((const void*)k_filter_line, bytes));
-    DGCT_TRY(raise_smem_limit((const void*)k_filter_pairs<float>, bytes));
-    DGCT_TRY(raise_smem_limit((const void*)k_filter_pairs<bf16s>, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_views<float>, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_views<bf16s>, bytes));
     DGCT_TRY(raise_smem_limit((const void*)k_img_rows_fwd, bytes));
     // several columns a block up to m = 2048: 4 at 1024 and 2 at 2048 need the same 74 KB
     DGCT_TRY(raise_smem_limit((const void*)k_img_cols,

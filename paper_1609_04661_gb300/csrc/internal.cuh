@@ -153,7 +153,6 @@ struct Workspace {
     float* zraw2 = nullptr;        // [M]  copy for in-place Toeplitz filtering
     float2* tw = nullptr;          // FFT twiddles for length P, stage by stage (fft_device.cuh)
     float2* tw2 = nullptr;         // the same for length m2
-    float2* twh = nullptr;         // the same for length P / 2 (H of a view as a real line)
     double* scratch_d = nullptr;   // plan-time FP64 scratch
     float* b = nullptr;            // the iteration's probe b (Eq. MC_SURE) [n][n]
     FanRay* fan_rays = nullptr;    // fan-beam plans: [n_views][n_det]
@@ -181,8 +180,7 @@ struct dgamp_ct_plan_s {
     int tv_rows = 64;                      // rows of a blocked TV region (32, 64 or 128)
     int tv_vrows = 4;                      // rows per thread of a TV region (4, or 8 with 64-row regions)
     int filter_mode = 0;                   // H by 0: FFT, 1: Toeplitz product (plan-time choice)
-    int filter_solve = 0;                  // the same inside a solve with exact moments (plan-time choice)
-    int filter_set = -1;                   // the form set by dgamp_ct_set_tuning for all of them (-1: none)
+    int filter_set = 0;                    // dgamp_ct_set_tuning has changed filter_mode
     int sino_fused = 0;                    // solve: H A x, output step, H s in one kernel (k_sino_step)
     int bp_mode = 0;                       // A^T: 0 pixel-driven gather, 1 ray-driven tiles (plan-time choice)
     int pj_seg = 8;                        // A: step segments (warps) per ray group, 8/16/32 (plan-time choice)
