@@ -511,14 +511,13 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
 // 130 activation pixels, a strip of 128 gradient pixels) feed the MMAs as they
 // land.
 //
-// All nine taps and the bias of an activation row take two MMAs per 16 pixels,
-// both M = 128, N = 192:
+// All nine taps of an activation row take two MMAs per 16 pixels, both M = 128,
+// N = 192:
 //   B = the gradient rows above, at and below the activation row (N = 3 x 64,
 //       one row slot apart; they are its dy = 2, 1 and 0 taps);
 //   A = the activation row twice, the second copy starting one pixel later
 //       (M = 2 x 64, the leading-dimension offset is one 128-byte row): dx = 0
-//       and 1; then once more from pixel 2, beside a block of ones: dx = 2 and,
-//       in the ones' rows, the gradient's own sums.
+//       and 1; then from pixel 2 (and 3, which nothing reads): dx = 2.
 // M = 64 halves fill half of the tensor core, and separate CTAs per dy read
 // both operands three times: that form took 25.5 us per layer on 32 patches of
 // 64 x 64 and two more kernels for the bias; this one takes
@@ -529,19 +528,22 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
 // error that grows with the number of additions, so after at most WG_CHAIN
 // steps of 16 pixels the sums move from tensor memory to the CTA's partial,
 // where one thread per element adds them up in FP32 (1e-5 relative without, at
-// 816 steps).  Warp 0 (one lane) loads rows, warp 1 issues the MMAs, warps 4..7
-// move the sums; gradient rows pass through a ring, and where three of them
+// 816 steps).  The bias sums, terms of one sign more often than the others', are
+// added in FP32 by two warps of their own from the gradient rows in shared memory:
+// rows of ones beside the third tap gave them for nothing, but cut off as above
+// they were up to 1.1e-6 of sum |g| away (16 images of 256 x 256, mean 1).  Warp 0
+// (one lane) loads rows, warp 1 issues the MMAs, warps 2 and 3 sum the bias, warps
+// 4..7 move the sums; gradient rows pass through a ring, and where three of them
 // wrap around its end the MMA is split in two.
 constexpr int WG_G_SLOT = M * 128;                     // 128 gradient pixels
 constexpr int WG_NA = 4, WG_NG = 6;                    // row slots of the two rings
-constexpr int WG_ONES = 2048;                          // 16 pixels x 64 ones
-constexpr int WG_SMEM = 1024 + WG_NA * A_ROW + WG_NG * WG_G_SLOT + WG_ONES;
+constexpr int WG_SMEM = 1024 + WG_NA * A_ROW + WG_NG * WG_G_SLOT;
 constexpr int WG_THREADS = 256;
 constexpr int WG_CHAIN = 320;                          // most accumulation steps (a row may start below, and end past it)
 constexpr unsigned WG_TMEM_COLS = 512;                 // two 192-column accumulators (a power of two)
 // One partial as it lies in tensor memory, [column][lane], so that a warp's lanes write whole lines.  Column
 // 64 r + co of the first accumulator: tap dy = 2 - r, dx = lane / 64, ci = lane % 64; of the second: lanes below 64
-// dx = 2, lane 64 of r = 1 the bias, the others nothing.
+// dx = 2.  Lane 64 of the second's columns 64 + co holds the bias; its other lanes from 64 on are not written.
 constexpr int WG_OUT = 2 * 192 * 128;
 // kind::f16 instruction descriptor: D FP32, A and B BF16, both MN-major, M = 128, N = 64 count
 __device__ __forceinline__ uint32_t idesc_wg(int count) { return idesc_n(count) | (1u << 15) | (1u << 16); }
@@ -569,6 +571,7 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     __shared__ __align__(8) uint64_t a_full[WG_NA], a_empty[WG_NA], g_full[WG_NG], g_empty[WG_NG];
     __shared__ __align__(8) uint64_t acc_full, acc_empty;
     __shared__ __align__(8) uint64_t never_bar;
+    __shared__ float bias_sum[2][CH];
     __shared__ uint32_t tmem_slot;
     __shared__ int stalled;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -576,7 +579,7 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     const int group = blockIdx.x, z = blockIdx.y;
     const int la = a_first - z, lg = g_first + g_step * z;    // layer slots of the two tensors
     const uint32_t raw = smem_u32(smem_raw);
-    const uint32_t sA = (raw + 1023u) & ~1023u, sG = sA + WG_NA * A_ROW, sOnes = sG + WG_NG * WG_G_SLOT;
+    const uint32_t sA = (raw + 1023u) & ~1023u, sG = sA + WG_NA * A_ROW;
     const int nx = (W + M - 1) / M;
     const int nstrips = B * H * nx;
     const int s0 = group * per;
@@ -599,7 +602,7 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         }
         for (int s = 0; s < WG_NG; ++s) {
             mbar_init(smem_u32(&g_full[s]), 1);
-            mbar_init(smem_u32(&g_empty[s]), 1);
+            mbar_init(smem_u32(&g_empty[s]), 3);     // the MMAs and the two bias warps
         }
         mbar_init(smem_u32(&acc_full), 1);
         mbar_init(smem_u32(&acc_empty), 4);
@@ -607,9 +610,6 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         stalled = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    for (int i = tid; i < WG_ONES / 4; i += WG_THREADS)      // BF16 1.0 pairs
-        asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(sOnes + 4 * i), "r"(0x3F803F80u) : "memory");
-    fence_async_smem();
     fence_before();
     __syncthreads();
     fence_after();
@@ -684,7 +684,7 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                     const uint32_t acc = (chain | ks) != 0 ? 1u : 0u;
                     const uint64_t go = (uint64_t)((ks * 16 * 128) >> 4);
                     const uint32_t at = a0 + (uint32_t)(ks * 16 * 128);
-                    const uint64_t a01 = sdesc_sw128_mn(at, 128u), a2 = sdesc_sw128_mn(at + 256u, sOnes - at - 256u);
+                    const uint64_t a01 = sdesc_sw128_mn(at, 128u), a2 = sdesc_sw128_mn(at + 256u, 128u);
                     mma_bf16(tmem, a01, g1 + go, i1, acc);
                     if (n2) mma_bf16(d2, a01, g2 + go, i2, acc);
                     mma_bf16(tmem + 192u, a2, g1 + go, i1, acc);
@@ -700,6 +700,55 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         }
         // arrives once every MMA issued above has completed
         mma_commit(smem_u32(&acc_full));
+    } else if (run && warp < 4 && warp >= 2) {
+        // ---- bias: each gradient row of the strips once; a thread takes 8 channels of every eighth pixel, adds a
+        // row's pixels apart and joins them to its total with Kahan's correction ----
+        const int t = tid - 64, chunk = t & 7, p0 = t >> 3;
+        const uint32_t at = sG + (uint32_t)(p0 * 128 + ((chunk ^ p0) * 16));      // swizzled as the TMA wrote it
+        float tot[8] = {}, corr[8] = {};
+        int qg = 0;
+        for (int s_a = s0; ok && s_a < s1;) {
+            const int R = run_end(s_a, s1, H) - s_a + 1, eights = 2 * wg_steps(s_a, H, W, nx);
+            for (int i = 0; i < R + 2; ++i, ++qg) {      // rows 0 and R + 1 lie outside the run
+                const int slot = qg % WG_NG;
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&g_full[slot]), (uint32_t)((qg / WG_NG) & 1)))) {
+                    ok = false;
+                    break;
+                }
+                if (i >= 1 && i <= R) {
+                    float row[8] = {};
+                    for (int j = 0; j < eights; ++j) {
+                        uint32_t v[4];
+                        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+                                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                                     : "r"(at + (uint32_t)(slot * WG_G_SLOT + j * 1024)));
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            row[2 * k] += __uint_as_float(v[k] << 16);
+                            row[2 * k + 1] += __uint_as_float(v[k] & 0xFFFF0000u);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float y = row[k] - corr[k], n = tot[k] + y;
+                        corr[k] = (n - tot[k]) - y;
+                        tot[k] = n;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&g_empty[slot])) : "memory");
+            }
+            s_a += R;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], 8);
+            tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], 16);
+            if (lane < 8) bias_sum[warp - 2][chunk * 8 + k] = tot[k];
+        }
+        named_bar(1, 64);
+        out[(256 + t) * 128 + 64] = bias_sum[0][t] + bias_sum[1][t];
     } else if (run && warp >= 4) {
         // ---- sums from tensor memory to the partial: stored the first time, then added (each element by
         // one thread, so in a fixed order) ----
@@ -720,7 +769,7 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                 __syncwarp();
                 tmem_ld32(tmem + lane_base + (uint32_t)(c * 32), v);   // warp-collective
                 asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-                if (c >= 6 && m >= 64 && !(m == 64 && (c == 8 || c == 9))) continue;
+                if (c >= 6 && m >= 64) continue;
                 float* dst = out + c * 32 * 128 + m;
                 if (flushes == 0) {
 #pragma unroll
@@ -838,8 +887,9 @@ int launch_conv64_tc(int mode, const void* in, const void* wk_all, int layers, i
 // Layers z = 0 .. nl - 1: input activations in slot a_first - z of `acts`,
 // output gradients in slot g_first + g_step z of `grads`, both
 // [slots][slot][64] BF16 with slot = slot_pix pixels of which the first B H W
-// are used; partial: [nl][groups][9 * 64 * 64 + 64] FP32, every one written
-// (zeros for a group without strips).
+// are used; partial: [nl][groups][wgrad64_partial_floats()] FP32 in the kernel's
+// [column][lane] layout, whose entries without a meaning are left unwritten
+// (a group without strips is all zeros).
 int wgrad64_partial_floats() { return tc::WG_OUT; }
 int launch_wgrad64_tc(const void* acts, int act_slots, int a_first, const void* grads, int grad_slots, int g_first,
                       int g_step, long long slot_pix, int nl, int B, int H, int W, int groups, float* partial,
