@@ -502,7 +502,6 @@ struct dgamp_ct_cnn_s {
     uint64_t ws_gen = 0;        // bumped whenever the workspace is reallocated or captured launches change
 };
 
-constexpr int kWgGroupsMax = 64;            // most CTA groups of the tensor-core weight gradient
 constexpr size_t kGradBytes = 1ull << 30;   // bound on the gradients kept for it
 
 static void cnn_free_ws(dgamp_ct_cnn_s* c) {
@@ -542,7 +541,7 @@ static int cnn_ensure_ws(dgamp_ct_cnn_s* c, int64_t npix, int nstore, int batch)
     if ((rc = A((void**)&c->f, (size_t)cap * sizeof(float))) != DGAMP_CT_OK) return rc;
     if ((rc = A((void**)&c->gout, (size_t)cap * sizeof(float))) != DGAMP_CT_OK) return rc;
     // the larger of the tensor-core weight gradient's partials and the pixel sums' (+ their reduction)
-    const size_t n_part = std::max((size_t)std::max(c->sm_count, kWgGroupsMax) * wgrad64_partial_floats(),
+    const size_t n_part = std::max((size_t)std::max(c->sm_count, c->L) * wgrad64_partial_floats(),
                                    (size_t)(kColBlocks + 1) * 10 * CH);
     if ((rc = A((void**)&c->partial, n_part * sizeof(float))) != DGAMP_CT_OK) return rc;
     if ((rc = A((void**)&c->dpart, 1024 * sizeof(double))) != DGAMP_CT_OK) return rc;
@@ -617,7 +616,7 @@ static int cnn_backward(dgamp_ct_cnn_s* c, const float* r, const float* sig, int
         for (int z = 0; z < nl; ++z, at += dir)
             DGCT_TRY(launch_conv64_tc(1, grad(at), c->wt, L - 2, l - z - 1, nullptr, act(l - z), grad(at + dir), B, H,
                                       W, c->sm_count, c->tc_err, st, c->stall_ns));
-        const int Gw = std::max(1, std::min(kWgGroupsMax, c->sm_count / nl));
+        const int Gw = std::max(1, c->sm_count / nl);
         DGCT_TRY(launch_wgrad64_tc(c->act, c->cap_store, l - 1, c->g, c->n_g, first, dir, c->cap_pix, nl, B, H, W, Gw,
                                    c->partial, c->tc_err, st, c->stall_ns));
         k_reduce_wgrad64<<<dim3((width + 255) / 256, nl), 256, 0, st>>>(c->partial, Gw, width, c->grad + c->w_off[l],
