@@ -530,14 +530,6 @@ static int cnn_ensure_ws(dgamp_ct_cnn_s* c, int64_t npix, int nstore, int batch)
     };
     int rc;
     if ((rc = A((void**)&c->act, (size_t)ns * cap * CH * sizeof(bf16))) != DGAMP_CT_OK) return rc;
-    // gradients of all layers where they fit kGradBytes, so that one launch takes every layer's
-    // weight gradient; else of as many as fit, and of two at least (as much as a layer by layer pass needs)
-    const size_t slot = (size_t)cap * CH * sizeof(bf16);
-    if (ns >= c->L - 1) {   // training
-        c->n_g = (int)std::min<size_t>(c->L - 1, std::max<size_t>(2, kGradBytes / slot));
-        if ((rc = A((void**)&c->g, c->n_g * slot)) == DGAMP_CT_ERR_OOM) rc = A((void**)&c->g, (c->n_g = 2) * slot);
-        if (rc != DGAMP_CT_OK) return rc;
-    }
     if ((rc = A((void**)&c->f, (size_t)cap * sizeof(float))) != DGAMP_CT_OK) return rc;
     if ((rc = A((void**)&c->gout, (size_t)cap * sizeof(float))) != DGAMP_CT_OK) return rc;
     // the larger of the tensor-core weight gradient's partials and the pixel sums' (+ their reduction)
@@ -547,6 +539,15 @@ static int cnn_ensure_ws(dgamp_ct_cnn_s* c, int64_t npix, int nstore, int batch)
     if ((rc = A((void**)&c->dpart, 1024 * sizeof(double))) != DGAMP_CT_OK) return rc;
     if ((rc = A((void**)&c->loss, sizeof(double))) != DGAMP_CT_OK) return rc;
     if ((rc = A((void**)&c->sig_buf, (size_t)cb * sizeof(float))) != DGAMP_CT_OK) return rc;
+    // gradients of all layers where they fit kGradBytes, so that one launch takes every layer's
+    // weight gradient; else of as many as fit, and of two at least (as much as a layer by layer pass
+    // needs).  Allocated last: the slots beyond two can be done without, the rest cannot
+    const size_t slot = (size_t)cap * CH * sizeof(bf16);
+    if (ns >= c->L - 1) {   // training
+        c->n_g = (int)std::min<size_t>(c->L - 1, std::max<size_t>(2, kGradBytes / slot));
+        if ((rc = A((void**)&c->g, c->n_g * slot)) == DGAMP_CT_ERR_OOM) rc = A((void**)&c->g, (c->n_g = 2) * slot);
+        if (rc != DGAMP_CT_OK) return rc;
+    }
     c->cap_pix = cap;
     c->cap_store = ns;
     c->cap_batch = cb;
