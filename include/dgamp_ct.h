@@ -219,9 +219,9 @@ typedef struct {
                              kernel h = IFFT_P(g) (no wrap-around since P >= 2 n_det).
                              The form of the single-step calls and of a solve's three
                              kernels, with one exception: a Laplace solve
-                             (output_moments = 0) told to run three kernels takes the FFT,
-                             as the fused form 1 does, until set_tuning has changed this
-                             field (setting the value that get reports changes nothing) */
+                             (output_moments = 0) told to run three kernels takes the FFT as
+                             the fused form 1 does, until set_tuning has changed this field
+                             to 1 (setting the value that get reports changes nothing) */
     int32_t tv_kb;        /* Chambolle steps per blocked TV launch, 1..10 */
     int32_t tv_rows;      /* rows of the image region one TV block holds: 32, 64 or 128
                              (the region is 64 columns wide) */

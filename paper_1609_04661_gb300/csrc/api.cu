@@ -22,7 +22,7 @@ int cuda_fail(cudaError_t e) {
 
 static void free_ws(Workspace& w) {
     void* ptrs[] = {w.XR, w.XC, w.x, w.r, w.b, w.p, w.zraw, w.z, w.s, w.hs, w.y, w.fft2d, w.partial,
-                    w.partial_div, w.S, w.log, w.vc, w.gain, w.tw, w.tw2, w.scratch_d, w.hx, w.zraw2,
+                    w.partial_div, w.S, w.log, w.vc, w.gain, w.tw, w.tw2, w.twh, w.twk, w.scratch_d, w.hx, w.zraw2,
                     w.fan_rays, w.fan_views, w.fan_gw, w.pj_order, w.pj_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -137,6 +137,8 @@ static int plan_alloc(dgamp_ct_plan_s* pl, const std::vector<double>& ang) {
     DGCT_TRY(dalloc(&w.gain, (size_t)pl->P));
     DGCT_TRY(dalloc(&w.tw, (size_t)fft_twiddle_count(pl->P) + 1));
     DGCT_TRY(dalloc(&w.tw2, (size_t)fft_twiddle_count(pl->m2) + 1));
+    DGCT_TRY(dalloc(&w.twh, (size_t)fft_twiddle_count(pl->P / 2) + 1));
+    DGCT_TRY(dalloc(&w.twk, (size_t)pl->P / 4 + 1));
     DGCT_TRY(dalloc(&w.hx, (size_t)2 * pl->nd));
     DGCT_TRY(dalloc(&w.zraw2, M));
     DGCT_TRY(dalloc(&w.scratch_d, (size_t)(pl->nd + 1) + 2 * pl->nd + pl->nv + (size_t)pl->nv * pl->nd));
@@ -202,6 +204,14 @@ static int plan_alloc(dgamp_ct_plan_s* pl, const std::vector<double>& ang) {
     };
     DGCT_TRY(twiddles(P, w.tw));
     DGCT_TRY(twiddles(pl->m2, w.tw2));
+    DGCT_TRY(twiddles(P / 2, w.twh));
+    std::vector<float4> wk(P / 4 + 1);      // exp(2 pi i k / P), cosine and sine in two parts each
+    for (int k = 0; k <= P / 4; ++k) {
+        const double c = std::cos(two_pi * k / P), s = std::sin(two_pi * k / P);
+        const float ch = (float)c, sh = (float)s;
+        wk[k] = make_float4(ch, sh, (float)(c - ch), (float)(s - sh));
+    }
+    DGCT_CUDA(cudaMemcpy(w.twk, wk.data(), wk.size() * sizeof(float4), cudaMemcpyHostToDevice));
 
     // ||Phi~||_F^2 on the device in FP64
     double* ang_dev = w.scratch_d + (pl->nd + 1) + 2 * pl->nd;

@@ -1,9 +1,8 @@
 // Shared-memory FFTs for the Radon preconditioner (Section 2.4, Eq. Aprecon).
 //
-//  * H on sinograms: one block filters two views at once, packed as the real
-//    and imaginary parts of one complex line.  Because the gain g is real and
-//    even, filtering a + i b gives H a + i H b, so one forward and one inverse
-//    complex FFT of length P serve two views.
+//  * H on sinograms: one block per view, the real line of length P as a complex
+//    one of length P/2 (even bins + i odd bins), split into the spectra of the
+//    even and odd bins for the gain and put together again.
 //  * V^-1 / V on images: a 2-D zero-padded FFT done as row FFTs, column FFTs
 //    with the radial gain applied between the forward and inverse column
 //    transforms, and inverse row FFTs.  It runs once per solve.
@@ -20,14 +19,97 @@ namespace dgct {
 static int fft_threads(int P) { return P / 8 < 32 ? 32 : (P / 8 > 512 ? 512 : P / 8); }
 
 // ------------------------------------------------------------ H on views --
-// Two views per block as one complex line of length P, which the real and even
-// gain filters both: the arithmetic of the fused sinogram kernel's FFT form.
-// (One view as a complex line of half the length was no faster, 52.6 against
-// 51.7 us for two filters and an output step at 90 x 1449 where runs differ by
-// 15%, and 4-5% further from 64 bits.)
+// One view per block.  With z[j] = x[2j] + i x[2j + 1] and Z its DFT of length
+// L = P / 2, the even and odd bins' DFTs are E = (Z[k] + conj Z[L-k]) / 2 and
+// O = (Z[k] - conj Z[L-k]) / 2i, and x's own are E +- w^k O at k and k + L,
+// w = exp(-2 pi i / P).  With these times the gains g[k] and g[k + L] = g[L-k] as
+// A and C, E' = (A + C) / 2 and O' = w^-k (A - C) / 2, and Z' = E' + i O' (at L-k:
+// conj E' + i conj O') transforms back to the filtered bins.  (Gathering E and O
+// by (g[k] +- g[L-k]) instead saves an addition each, but lets the high
+// frequencies' rounding into the low ones, which A^T then amplifies.)
+//
+// E - w^k O cancels at the low frequencies, where most of a sinogram lies, and the
+// gain then raises what is left of the roundings; so E, O, w^k and the products
+// keep their low parts up to that difference (filter_split).  Against 64 bits H is
+// then as close as by two views in one complex line of length P (k_filter_pairs;
+// 0.98-1.0 of its error over 24 geometries), where plain FP32 was 4-5% off it.
+// The block's chain of stages and barriers bounds the kernel, not its arithmetic:
+// 64 x 729 takes 5.8 us with or without the low parts, pairs of views 9.0;
+// 90 x 1449 7.3 against 12.1.
+struct TwoPart {
+    float hi, lo;
+};
+__device__ __forceinline__ TwoPart two_sum(float a, float b) {      // Knuth: hi + lo = a + b exactly
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+
+// E + d and E - d for d = c a + s b, c and s in two parts (w.x + w.z, w.y + w.w)
+__device__ __forceinline__ void add_and_subtract(TwoPart E, TwoPart a, TwoPart b, float c, float s, float cl, float sl,
+                                                 float& plus, float& minus) {
+    const float p = __fmul_rn(c, a.hi), q = __fmul_rn(s, b.hi);
+    const TwoPart d = two_sum(p, q);
+    float lo = fmaf(c, a.hi, -p) + fmaf(s, b.hi, -q) + d.lo;
+    lo = fmaf(c, a.lo, fmaf(s, b.lo, fmaf(cl, a.hi, fmaf(sl, b.hi, lo))));
+    plus = __fadd_rn(__fadd_rn(E.hi, d.hi), E.lo + lo);
+    minus = __fadd_rn(__fsub_rn(E.hi, d.hi), E.lo - lo);
+}
+
+// 2 (E + w^k O) and 2 (E - w^k O) from Z[k] and Z[L-k]; w = exp(2 pi i k / P) in two parts
+__device__ __forceinline__ void filter_split(float2 z, float2 y, float4 w, float2& plus, float2& minus) {
+    const TwoPart Ex = two_sum(z.x, y.x), Ey = two_sum(z.y, -y.y), Ox = two_sum(z.y, y.y), Oy = two_sum(y.x, -z.x);
+    add_and_subtract(Ex, Ox, Oy, w.x, w.y, w.z, w.w, plus.x, minus.x);
+    add_and_subtract(Ey, Oy, Ox, w.x, -w.y, w.z, -w.w, plus.y, minus.y);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(512)
-k_filter_views(const T* in, T* out, int nv, int nd, int P,
+k_filter_line(const T* in, T* out, int nd, int P, const float* __restrict__ gain, const float2* __restrict__ tw,
+              const float4* __restrict__ wk) {
+    extern __shared__ float2 smem[];
+    const int L = P >> 1;
+    float2* a = smem;
+    float2* b = smem + fft_buf_len(L);
+    const T* row = in + (size_t)blockIdx.x * nd;
+    pdl_wait();
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
+        float2 v = make_float2(0.f, 0.f);
+        if (2 * i < nd) v.x = ldf(row + 2 * i);
+        if (2 * i + 1 < nd) v.y = ldf(row + 2 * i + 1);
+        a[fpad(i)] = v;
+    }
+    __syncthreads();
+    float2* r = fft_stockham(a, b, L, tw, -1.f);
+    float2* o = (r == a) ? b : a;
+    const float sc = 0.25f / (float)L;      // the two halvings above, and 1 / L of the inverse
+    for (int k = threadIdx.x; k <= L / 2; k += blockDim.x) {
+        const int kk = (L - k) & (L - 1);
+        const float2 z = r[fpad(k)], y = r[fpad(kk)];
+        const float ga = __ldg(gain + k) * sc, gb = __ldg(gain + L - k) * sc;
+        const float4 w = wk[k];                                                                      // w^-k
+        float2 A, C;
+        filter_split(z, y, w, A, C);
+        A = make_float2(ga * A.x, ga * A.y);
+        C = make_float2(gb * C.x, gb * C.y);
+        const float2 e = cadd(A, C), q = cmul(csub(A, C), make_float2(w.x, w.y));
+        r[fpad(k)] = make_float2(e.x - q.y, e.y + q.x);
+        if (kk != k) r[fpad(kk)] = make_float2(e.x + q.y, q.x - e.y);
+    }
+    __syncthreads();
+    r = fft_stockham(r, o, L, tw, 1.f);
+    T* w = out + (size_t)blockIdx.x * nd;
+    for (int i = threadIdx.x; i < nd; i += blockDim.x) {
+        const float2 v = r[fpad(i >> 1)];
+        stf(w + i, (i & 1) ? v.y : v.x);
+    }
+}
+
+// Two views per block as one complex line of length P, which the real and even
+// gain filters both: the arithmetic of the fused sinogram kernel's FFT form, for
+// Laplace solves that run it as a kernel of its own (filter_form).
+template <typename T>
+__global__ void __launch_bounds__(512)
+k_filter_pairs(const T* in, T* out, int nv, int nd, int P,
                const float* __restrict__ gain, const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
     float2* a = smem;
@@ -133,44 +215,49 @@ static size_t toeplitz_smem(int nd) {
 }
 
 // H's form for launch_filter.  The single steps, and a solve with exact moments,
-// take the plan's timed choice.  A Laplace solve runs the three kernels only if
-// told to (sino_fused = 0), beside the fused FFT form, and takes the FFT as well
-// unless the tuning has set a form: then the two forms agree bit for bit, where
-// the Toeplitz product's order of summation parts them by up to 1.5e-4 in tau_r
-// over five iterations of a 16 x 16 image (3 views of 24 bins).
-static bool filter_by_toeplitz(const dgamp_ct_plan_s* pl, int solve) {
-    if (solve && !pl->opt.output_moments && !pl->filter_set) return false;
-    return pl->filter_mode == 1;
+// take the plan's timed choice between the line per view and the Toeplitz product.
+// A Laplace solve runs the three kernels only if told to (sino_fused = 0), beside
+// the fused FFT form, and takes that form's arithmetic unless the tuning has set
+// the Toeplitz product: the two then agree bit for bit, where another order of
+// summation parts them by up to 1.6e-4 in tau_r over five iterations of a 16 x 16
+// image (3 views of 24 bins).
+enum FilterForm { kFilterLine, kFilterPairs, kFilterToeplitz };
+static FilterForm filter_form(const dgamp_ct_plan_s* pl, int solve) {
+    const bool laplace = solve && !pl->opt.output_moments;
+    if (pl->filter_mode == 1 && (!laplace || pl->filter_set)) return kFilterToeplitz;
+    return laplace ? kFilterPairs : kFilterLine;
+}
+
+template <typename T>
+static int launch_filter_t(const dgamp_ct_plan_s* pl, FilterForm form, const T* in, T* out, cudaStream_t st) {
+    const int P = pl->P;
+    if (form == kFilterToeplitz) {
+        // the block reads its whole input row first, so in == out needs a copy
+        const T* src = in;
+        if (in == out) {
+            DGCT_CUDA(cudaMemcpyAsync(pl->ws.zraw2, in, (size_t)pl->M * sizeof(T), cudaMemcpyDeviceToDevice, st));
+            src = (const T*)pl->ws.zraw2;
+        }
+        DGCT_CUDA(launch_pdl(k_filter_toeplitz<T>, dim3((pl->nd + kTzOut - 1) / kTzOut, pl->nv), dim3(32 * kTzWarps),
+                             toeplitz_smem(pl->nd), st, src, out, pl->nd, pl->ws.hx));
+        return DGAMP_CT_OK;
+    }
+    if (form == kFilterPairs) {
+        DGCT_CUDA(launch_pdl(k_filter_pairs<T>, dim3((pl->nv + 1) / 2), dim3(fft_threads(P)),
+                             (size_t)2 * fft_buf_len(P) * sizeof(float2), st, in, out, pl->nv, pl->nd, P, pl->ws.gain,
+                             pl->ws.tw));
+        return DGAMP_CT_OK;
+    }
+    DGCT_CUDA(launch_pdl(k_filter_line<T>, dim3(pl->nv), dim3(fft_threads(P / 2)),
+                         (size_t)2 * fft_buf_len(P / 2) * sizeof(float2), st, in, out, pl->nd, P, pl->ws.gain,
+                         pl->ws.twh, pl->ws.twk));
+    return DGAMP_CT_OK;
 }
 
 // bf = 1: in and out hold BF16 (a solve with storage = 1); sums in FP32 either way
 int launch_filter(const dgamp_ct_plan_s* pl, const float* in, float* out, cudaStream_t st, int bf, int solve) {
-    if (filter_by_toeplitz(pl, solve)) {
-        // the block reads its whole input row first, so in == out needs a copy
-        const float* src = in;
-        if (in == out) {
-            DGCT_CUDA(cudaMemcpyAsync(pl->ws.zraw2, in, (size_t)pl->M * (bf ? 2 : 4), cudaMemcpyDeviceToDevice, st));
-            src = pl->ws.zraw2;
-        }
-        const dim3 grd((pl->nd + kTzOut - 1) / kTzOut, pl->nv), blk(32 * kTzWarps);
-        const size_t sm = toeplitz_smem(pl->nd);
-        if (bf)
-            DGCT_CUDA(launch_pdl(k_filter_toeplitz<bf16s>, grd, blk, sm, st, (const bf16s*)src, (bf16s*)out, pl->nd,
-                                 pl->ws.hx));
-        else
-            DGCT_CUDA(launch_pdl(k_filter_toeplitz<float>, grd, blk, sm, st, src, out, pl->nd, pl->ws.hx));
-        return DGAMP_CT_OK;
-    }
-    const int P = pl->P;
-    const size_t sm = (size_t)2 * fft_buf_len(P) * sizeof(float2);
-    const dim3 grd((pl->nv + 1) / 2), blk(fft_threads(P));
-    if (bf)
-        DGCT_CUDA(launch_pdl(k_filter_views<bf16s>, grd, blk, sm, st, (const bf16s*)in, (bf16s*)out, pl->nv, pl->nd, P,
-                             pl->ws.gain, pl->ws.tw));
-    else
-        DGCT_CUDA(launch_pdl(k_filter_views<float>, grd, blk, sm, st, in, out, pl->nv, pl->nd, P, pl->ws.gain,
-                             pl->ws.tw));
-    return DGAMP_CT_OK;
+    const FilterForm form = filter_form(pl, solve);
+    return bf ? launch_filter_t(pl, form, (const bf16s*)in, (bf16s*)out, st) : launch_filter_t(pl, form, in, out, st);
 }
 
 // Plan-time choice between the FFT and the Toeplitz form of H (same operator):
@@ -313,8 +400,10 @@ int launch_precond_images(const dgamp_ct_plan_s* pl, const float* in, float* out
 }
 
 int fft_set_smem_limits(int bytes) {
-    DGCT_TRY(raise_smem_limit((const void*)k_filter_views<float>, bytes));
-    DGCT_TRY(raise_smem_limit((const void*)k_filter_views<bf16s>, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_line<float>, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_line<bf16s>, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_pairs<float>, bytes));
+    DGCT_TRY(raise_smem_limit((const void*)k_filter_pairs<bf16s>, bytes));
     DGCT_TRY(raise_smem_limit((const void*)k_img_rows_fwd, bytes));
     // several columns a block up to m = 2048: 4 at 1024 and 2 at 2048 need the same 74 KB
     DGCT_TRY(raise_smem_limit((const void*)k_img_cols,

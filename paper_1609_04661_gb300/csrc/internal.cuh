@@ -153,6 +153,8 @@ struct Workspace {
     float* zraw2 = nullptr;        // [M]  copy for in-place Toeplitz filtering
     float2* tw = nullptr;          // FFT twiddles for length P, stage by stage (fft_device.cuh)
     float2* tw2 = nullptr;         // the same for length m2
+    float2* twh = nullptr;         // the same for length P / 2 (H of a view as a real line)
+    float4* twk = nullptr;         // [P / 4 + 1]  exp(2 pi i k / P) in two parts
     double* scratch_d = nullptr;   // plan-time FP64 scratch
     float* b = nullptr;            // the iteration's probe b (Eq. MC_SURE) [n][n]
     FanRay* fan_rays = nullptr;    // fan-beam plans: [n_views][n_det]
@@ -179,7 +181,7 @@ struct dgamp_ct_plan_s {
     int tv_kb = 5;                         // Chambolle steps per blocked TV launch
     int tv_rows = 64;                      // rows of a blocked TV region (32, 64 or 128)
     int tv_vrows = 4;                      // rows per thread of a TV region (4, or 8 with 64-row regions)
-    int filter_mode = 0;                   // H by 0: FFT, 1: Toeplitz product (plan-time choice)
+    int filter_mode = 0;                   // H by 0: FFT, 1: Toeplitz product (plan-time choice; filter_form in fft.cu)
     int filter_set = 0;                    // dgamp_ct_set_tuning has changed filter_mode
     int sino_fused = 0;                    // solve: H A x, output step, H s in one kernel (k_sino_step)
     int bp_mode = 0;                       // A^T: 0 pixel-driven gather, 1 ray-driven tiles (plan-time choice)
