@@ -36,6 +36,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "internal.cuh"
@@ -525,10 +526,13 @@ k_conv64_tc(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ 
 //
 // One launch covers several layers (blockIdx.y): each CTA sums its layer over a
 // contiguous range of strips.  The tensor core truncates as it accumulates, an
-// error that grows with the number of additions, so after at most WG_CHAIN
-// steps of 16 pixels the sums move from tensor memory to the CTA's partial,
+// error that grows with the number of additions, so after a fiftieth of a layer's
+// steps of 16 pixels (WG_SHARES: as many chains as a launch of one layer had CTAs
+// per tap row), and WG_CHAIN at most, the sums move from tensor memory to the CTA's partial,
 // where one thread per element adds them up in FP32 (1e-5 relative without, at
-// 816 steps).  The bias sums, terms of one sign more often than the others', are
+// 816 steps).  Sums of one sign on 32 patches of 64 x 64 are then 3.5e-7 off, with
+// WG_CHAIN alone 9.0e-7, for 1% of the pass (833 against 826 us; 3% on 8 patches).
+// The bias sums, terms of one sign more often than the others', are
 // added in FP32 by two warps of their own from the gradient rows in shared memory:
 // rows of ones beside the third tap gave them for nothing, but cut off as above
 // they were up to 1.1e-6 of sum |g| away (16 images of 256 x 256, mean 1).  Warp 0
@@ -540,6 +544,7 @@ constexpr int WG_NA = 4, WG_NG = 6;                    // row slots of the two r
 constexpr int WG_SMEM = 1024 + WG_NA * A_ROW + WG_NG * WG_G_SLOT;
 constexpr int WG_THREADS = 256;
 constexpr int WG_CHAIN = 320;                          // most accumulation steps (a row may start below, and end past it)
+constexpr int WG_SHARES = 50;                          // chains a layer's pixels are cut into at least
 constexpr unsigned WG_TMEM_COLS = 512;                 // two 192-column accumulators (a power of two)
 // One partial as it lies in tensor memory, [column][lane], so that a warp's lanes write whole lines.  Column
 // 64 r + co of the first accumulator: tap dy = 2 - r, dx = lane / 64, ci = lane % 64; of the second: lanes below 64
@@ -565,7 +570,7 @@ __device__ __forceinline__ uint64_t sdesc_sw128_mn(uint32_t saddr, uint32_t lbo)
 
 __global__ void __launch_bounds__(WG_THREADS, 1)
 k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_g, int a_first,
-             int g_first, int g_step, int B, int H, int W, int per, float* __restrict__ partial, unsigned* err,
+             int g_first, int g_step, int B, int H, int W, int per, int chain_max, float* __restrict__ partial, unsigned* err,
              unsigned long long stall_ns) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t a_full[WG_NA], a_empty[WG_NA], g_full[WG_NG], g_empty[WG_NG];
@@ -660,7 +665,7 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             const int nks = wg_steps(s_a, H, W, nx);
             for (int i = 0; i <= s_e - s_a; ++i, ++qa, ++qg) {
                 bool got = true;
-                if (chain >= WG_CHAIN) {
+                if (chain >= chain_max) {
                     mma_commit(smem_u32(&acc_full));
                     got = mbar_wait(smem_u32(&acc_empty), (uint32_t)(flushes & 1));
                     ++flushes;
@@ -757,7 +762,7 @@ k_wgrad64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         int chain = 0, flushes = 0;
         for (int s = s0; s < s1; ++s) {
             chain += wg_steps(s, H, W, nx);
-            if (chain < WG_CHAIN && s + 1 < s1) continue;
+            if (chain < chain_max && s + 1 < s1) continue;
             if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full), (uint32_t)(flushes & 1)))) {
                 ok = false;
                 break;
@@ -913,8 +918,12 @@ int launch_wgrad64_tc(const void* acts, int act_slots, int a_first, const void* 
         DGCT_TRY(encode(&map_g, 5, grads, dims, strides, box));
     }
     const int per = (int)((nstrips + groups - 1) / groups);
+    long long steps = 0;      // of a layer: 16 pixels each
+    for (int x = 0; x < W; x += tc::M) steps += (std::min(W - x, tc::M) + 15) / 16;
+    steps *= (long long)B * H;
+    const int chain_max = (int)std::min<long long>(tc::WG_CHAIN, (steps + tc::WG_SHARES - 1) / tc::WG_SHARES);
     tc::k_wgrad64_tc<<<dim3(groups, nl), tc::WG_THREADS, tc::WG_SMEM, st>>>(map_a, map_g, a_first, g_first, g_step, B, H,
-                                                                           W, per, partial, err, stall_ns);
+                                                                           W, per, chain_max, partial, err, stall_ns);
     DGCT_LAUNCH_CHECK();
     return DGAMP_CT_OK;
 }
