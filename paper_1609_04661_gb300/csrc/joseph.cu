@@ -448,7 +448,8 @@ k_backproject(const T* __restrict__ sino, int nv, int nd, int n,
 // accumulator tiles gave (24 geometries of 64^2 .. 1024^2, 0.74 .. 0.97; 1.01 with
 // the views in sequence, 1.2 with the mantissa's weights and one chain of sums).
 // Per iteration of the 512^2/64/729 solve about 30.7 -> 16 us; one call at
-// 1024^2/90/1449 124 -> about 59 us, of which the order of the views takes 1.
+// 1024^2/90/1449 124 -> 51 us (back to back).  A view's place in the sinogram is
+// staged with its constants: formed at each load from the slot, it cost 2 us there.
 // What is left is issue (half of the cycles) and the set-up and staging of blocks
 // that all start at once.  8 blocks per SM: 10 spill, 6 are slower.
 constexpr int kBtS = 16;
@@ -466,6 +467,7 @@ struct BtShared {
     int4 vc[kBtViews];           // position of pixel (8, 8), its steps along x and y, and A per position unit
     float om[kBtViews];          // 1 - A
     float2 low[kBtViews];        // first staged ray (int bits), path length per step
+    int row[kBtViews];           // the first staged ray's place in the sinogram
     unsigned s_max;
     float s_tau_r;
 };
@@ -480,14 +482,15 @@ __device__ __forceinline__ int bt_view(int i, int cnt) {
 }
 
 // Constants of views v0 .. v0 + cnt - 1 for the tile at (tx0, ty0).
-__device__ __forceinline__ void bt_view_setup(const ViewConst* __restrict__ vcs, int v0, int cnt, int tx0, int ty0,
-                                              BtShared& sh) {
+__device__ __forceinline__ void bt_view_setup(const ViewConst* __restrict__ vcs, int v0, int cnt, int nd, int tx0,
+                                              int ty0, BtShared& sh) {
     for (int i = threadIdx.x; i < kBtViews; i += kBtWork) {
         const int k = bt_view(i, cnt);
         if (k >= cnt) {              // pads the partial sums: no rays, all values 0
             sh.vc[i] = make_int4(0, 0, 0, 0);
             sh.om[i] = 0.f;
             sh.low[i] = make_float2(__int_as_float(INT_MIN / 2), 0.f);
+            sh.row[i] = 0;
             continue;
         }
         const ViewConst& c = vcs[v0 + k];
@@ -503,6 +506,7 @@ __device__ __forceinline__ void bt_view_setup(const ViewConst* __restrict__ vcs,
                              __float_as_int(A * (1.f / (float)(1 << kBtFrac))));      // exact: a power of two
         sh.om[i] = 1.f - A;
         sh.low[i] = make_float2(__int_as_float((int)lo), c.w);
+        sh.row[i] = (v0 + k) * nd + (int)lo;
     }
 }
 
@@ -512,7 +516,7 @@ __device__ __forceinline__ void bt_view_setup(const ViewConst* __restrict__ vcs,
 // trip the blocks, which all start at once, spent as long here as in the sums.
 constexpr int kBtBatch = 8;
 template <typename T>
-__device__ __forceinline__ bool bt_stage(const T* __restrict__ sino, int v0, int cnt, int nd, BtShared& sh) {
+__device__ __forceinline__ bool bt_stage(const T* __restrict__ sino, int cnt, int nd, BtShared& sh) {
     const int lane = threadIdx.x & 31;
     constexpr int nw = kBtWork / 32;
     const int pad = (cnt + kBtUnroll - 1) / kBtUnroll * kBtUnroll;
@@ -523,9 +527,8 @@ __device__ __forceinline__ bool bt_stage(const T* __restrict__ sino, int v0, int
         for (int k = 0; k < kBtBatch; ++k) {
             const int i = min(i0 + nw * k, kBtViews - 1);
             const float2 lw = sh.low[i];
-            const int d = __float_as_int(lw.x) + lane;
             v[k] = 0.f;
-            if ((unsigned)d < (unsigned)nd) v[k] = ldf(sino + (size_t)(v0 + bt_view(i, cnt)) * nd + d) * lw.y;
+            if ((unsigned)(__float_as_int(lw.x) + lane) < (unsigned)nd) v[k] = ldf(sino + (sh.row[i] + lane)) * lw.y;
         }
 #pragma unroll
         for (int k = 0; k < kBtBatch; ++k) {
@@ -608,7 +611,7 @@ __device__ __forceinline__ void backproject_tile_block(const T* __restrict__ sin
         pdl_wait();
         bp_tau_r(S, partial, nparts, M, (double)n * n, &sh.s_tau_r, first);
     } else {
-        bt_view_setup(vcs, 0, min(nv, kBtViews), tx0, ty0, sh);            // plan constants: before the wait
+        bt_view_setup(vcs, 0, min(nv, kBtViews), nd, tx0, ty0, sh);            // plan constants: before the wait
         pdl_wait();      // H s and the tau_s partials are the previous kernel's output
         if (update && ix < n)
 #pragma unroll
@@ -618,10 +621,10 @@ __device__ __forceinline__ void backproject_tile_block(const T* __restrict__ sin
             const int cnt = min(kBtViews, nv - v0);
             if (v0 > 0) {
                 bt_sync();                                                 // the previous views are done with
-                bt_view_setup(vcs, v0, cnt, tx0, ty0, sh);
+                bt_view_setup(vcs, v0, cnt, nd, tx0, ty0, sh);
             }
             bt_sync();
-            const bool bad = bt_stage(sino, v0, cnt, nd, sh);
+            const bool bad = bt_stage(sino, cnt, nd, sh);
             if (bt_sync_or(bad))
                 bt_views<true>(sh, cnt, lx, ly, acc0, acc1);
             else
