@@ -17,7 +17,8 @@
  *    unless explicit angles are given; ray (theta, u) is the line
  *    X cos(theta) + Y sin(theta) = u.
  *  - A is Joseph's ray-driven linear-interpolation projector (Eq. linCT's
- *    a_ij, which the paper leaves to a toolbox); A^T is its exact transpose.
+ *    a_ij, which the paper leaves to a toolbox); A^T is its transpose, exactly
+ *    or to the rounding of the weights (dgamp_ct_tuning, bp_mode).
  *  - H is the detector-axis form of the preconditioner: per view, zero-pad to
  *    P = smallest power of two >= 2 n_det, FFT, multiply by
  *    g_k = sqrt(max(|k/P|, 1/(2P))) (signed frequency), inverse FFT, crop.
@@ -238,8 +239,13 @@ typedef struct {
                              1 = 16 x 16 image tiles that stage the rays of 64 views in
                              shared memory and evaluate the weights from each pixel's
                              detector coordinate (within 2^-22 of the projector's).  Both
-                             are the projector's transpose and deterministic; a fan-beam
-                             plan's form 1 is ray-driven, with the projector's weights */
+                             are the projector's transpose and deterministic.  Fan beam:
+                             0 = the gather, 1 = the tiles, where the rays of a view allow
+                             a lane stride without conflicts: pixel by pixel as above where
+                             rays lie 1/2 to 3 pixels apart in the image and a tile's rays
+                             fit its buffer (weights from 26-bit positions, A^T s within
+                             about 1e-7 as from the projector's), else ray by ray with the
+                             projector's weights */
     int32_t pj_seg;       /* A: warps that split the step range of one group of 32 rays,
                              8, 16 or 32 (the partial sums are added in a fixed order) */
     int32_t tv_vrows;     /* rows of the TV region each thread holds: 4; 8 or 2 (then the

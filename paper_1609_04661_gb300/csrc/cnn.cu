@@ -15,9 +15,9 @@
 //
 // The 64 -> 64 layers (forward, input gradient and forward-mode tangent) are
 // implicit GEMMs on the tcgen05 tensor cores with TMEM accumulators
-// (conv_tc.cu), and so is their weight gradient (M = 64 co, N = 64 ci per
-// tap, K = pixels), which writes per-CTA FP32 partials that a second kernel
-// adds in a fixed order.  The first (1 -> 64) and last
+// (conv_tc.cu), and so is their weight gradient (M = 128: ci of two taps of a
+// row, N = 192: co of three rows, K = pixels), which writes per-CTA FP32 partials
+// that a second kernel adds in a fixed order.  The first (1 -> 64) and last
 // (64 -> 1) layers are small and run on the CUDA cores.
 #include <cuda_bf16.h>
 

@@ -86,10 +86,9 @@ constexpr uint32_t IDESC0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(M >
 __device__ __forceinline__ uint32_t idesc_n(int count) { return IDESC0 | ((uint32_t)(count * (64 >> 3)) << 17); }
 
 // Called by a whole converged warp; elect.sync picks the one lane that issues
-// (always the same one, so its commits cover its MMAs).  With warp-uniform
-// control flow the operands stay in uniform registers: issued from a branch
-// that only lane 0 takes, the operands are moved there one by one and an MMA
-// took 146 cycles to issue, more than it takes to execute.
+// (always the same one, so its commits cover its MMAs).  Issued from a branch
+// that only lane 0 takes, an MMA took 146 cycles to issue, more than it takes to
+// execute; from the converged warp they issue at the rate they execute.
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                          uint32_t accumulate) {
     asm volatile(

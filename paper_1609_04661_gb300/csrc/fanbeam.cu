@@ -1,5 +1,5 @@
 // Flat-detector fan beam (Section 6; option of the plan, dgamp_ct_plan_fan):
-// the Joseph projector A along each ray's own direction, its exact
+// the Joseph projector A along each ray's own direction, its
 // transpose, and ||Phi~||_F^2 for Phi~ = A V^-1 (Eq. precondAMP_op with the
 // image-domain cone filter; the detector-axis form H A is a parallel-beam
 // identity and does not apply).
@@ -13,8 +13,8 @@
 // linear interpolation between the two nearest rows is weighted by
 // w = |v| / |v_x|; any other ray is marched by rows with the fractional
 // column a0 + s a_step, a_step = -v_x / v_y, w = |v| / |v_y|.  Positions are
-// 32.32 fixed point computed once per ray in FP64, so the projector and the
-// back-projector take bit-identical taps.
+// 32.32 fixed point computed once per ray in FP64; the projector and the
+// ray-driven and gather forms of the back-projector take bit-identical taps.
 //
 // A: one block = 32 adjacent rays of one view; 8 warps march disjoint parts
 // of the step range and add their partial sums in a fixed order.  A ray
@@ -22,9 +22,13 @@
 // marched by rows the staged rows XR, as in joseph.cu; taps just outside the
 // image read the zero guard cells.
 //
-// A^T, ray-driven tiles (bp_mode 1, the default where it applies): one
-// block = one 16 x 16 image tile, warp w takes views w, w + 8, ...  The rays
-// of a view that can put a tap in the tile are those whose bins lie between
+// A^T, tiles pixel by pixel (bp_mode 1 where fan_gather_ok holds, as at a
+// scanner's proportions): k_fan_backproject_gather below, whose weights come from
+// the pixel's detector coordinate.
+//
+// A^T, ray-driven tiles (bp_mode 1 elsewhere, the default where a lane stride
+// exists): one block = one 16 x 16 image tile, warp w takes views w, w + 8, ...
+// The rays of a view that can put a tap in the tile are those whose bins lie between
 // the bins of the corners of the tile grown by one pixel (the bin map is
 // monotone along any segment in front of the source, so its extremes over
 // the square are at the corners), widened by one bin each way.  A warp's 32

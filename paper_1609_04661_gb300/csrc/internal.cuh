@@ -184,7 +184,7 @@ struct dgamp_ct_plan_s {
     int filter_mode = 0;                   // H by 0: FFT, 1: Toeplitz product (plan-time choice; filter_form in fft.cu)
     int filter_set = 0;                    // dgamp_ct_set_tuning has changed filter_mode
     int sino_fused = 0;                    // solve: H A x, output step, H s in one kernel (k_sino_step)
-    int bp_mode = 0;                       // A^T: 0 pixel-driven gather, 1 ray-driven tiles (plan-time choice)
+    int bp_mode = 0;                       // A^T: 0 pixel-driven gather, 1 tiles (plan-time choice)
     int pj_seg = 8;                        // A: step segments (warps) per ray group, 8/16/32 (plan-time choice)
     int pj_band = 0;                       // A: 0 ray-group form; 16 or 32: lines per shared-memory band
     int pj_waves = 1;                      // A, banded form: full waves of blocks (1 or 2)

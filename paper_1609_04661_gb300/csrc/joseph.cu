@@ -1,4 +1,4 @@
-// Joseph ray-driven projector A, its exact transpose A^T, and the plan-time
+// Joseph ray-driven projector A, its transpose A^T, and the plan-time
 // FP64 evaluation of ||Phi~||_F^2 (Eq. linCT; Algorithm 1, Steps 1 and 3).
 //
 // Layout.  Before a projection the image is staged twice in row-padded form:
